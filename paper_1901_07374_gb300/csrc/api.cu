@@ -385,6 +385,35 @@ DevMat make_dev_mat(const tlsph_material &m)
     return d;
 }
 
+// The pair table of an FP64 context in library-owned memory, formed once every
+// material it uses is set and again when one is set anew (its entries hold
+// Young's moduli).  32 bytes a pair: 0.8 GB for 256,000 particles.  It is left
+// out (the steps then form the terms in place) where it would take more than a
+// quarter of the free device memory, so that it never decides how many
+// contexts fit.
+static cudaError_t ctx_pair_table(tlsph_ctx *ctx)
+{
+    if (ctx->cfg.precision != TLSPH_PRECISION_FP64 || !ctx->owns_mem || ctx->nnz == 0) return cudaSuccess;
+    for (int k = 0; k < TLSPH_MAX_MATERIALS; ++k)
+        if (ctx->mat_used[k] && !ctx->mat_set[k]) return cudaSuccess;
+    const size_t tab = (size_t)ctx->nnz * sizeof(double4_32a), bytes = tab + 3 * (size_t)ctx->N * sizeof(double);
+    if (!ctx->ptab_mem) {
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || bytes > avail / 4 ||
+            cudaMalloc(&ctx->ptab_mem, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->ptab_mem = nullptr;
+            return cudaSuccess;
+        }
+    }
+    double *S0 = reinterpret_cast<double *>(static_cast<char *>(ctx->ptab_mem) + tab);
+    const cudaError_t e = build_pair_table(ctx->s, ctx->cfg.h, static_cast<double4_32a *>(ctx->ptab_mem), S0, ctx->stream);
+    if (e != cudaSuccess) return e;
+    ctx->s.ptab = static_cast<const double4_32a *>(ctx->ptab_mem);
+    ctx->s.ps0 = S0;
+    return cudaSuccess;
+}
+
 // The per-slot weight table of pass-1 plan form 5 (library-owned memory;
 // 4 bytes per slot): slice offsets from the slice widths on the host, the
 // weights by k_w1t_fill.  Released again when a plan without it is set.
@@ -720,6 +749,8 @@ int tlsph_set_material(tlsph_ctx *ctx, int mat_id, const tlsph_material *m)
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set_material copy");
     e = launch_material_fields(ctx->s, mat_id, ctx->dcur, ctx->steps == 0, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set_material fields");
+    e = ctx_pair_table(ctx);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "pair table");
     // the copy source lives in ctx; wait so a later overwrite cannot race it
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set_material sync");
@@ -1069,6 +1100,7 @@ int tlsph_destroy(tlsph_ctx *ctx)
     if (ctx->w1t_mem) cudaFree(ctx->w1t_mem);
     if (ctx->w1t_off_mem) cudaFree(ctx->w1t_off_mem);
     if (ctx->col_mem) cudaFree(ctx->col_mem);
+    if (ctx->ptab_mem) cudaFree(ctx->ptab_mem);
     for (auto &ev : ctx->prof_ev) cudaEventDestroy(ev);
     mixed_release(*ctx);
     delete ctx;

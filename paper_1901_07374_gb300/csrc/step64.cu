@@ -12,16 +12,21 @@
 // plus hourglass control, then the velocity-Verlet update with the
 // velocity constraints and the fully damaged particles held at rest.
 //
-// Work decomposition: a warp owns 32 consecutive rows.  For each of them the
-// 32 lanes stride over the row's neighbours and the partial sums meet in a
-// butterfly reduction; lane r keeps row r's sums.  The per-particle epilogue
-// then runs on all 32 lanes at once, one particle per lane, so the heavy
-// FP64 constitutive work never leaves lanes idle.  Sums over j are therefore
-// grouped by lane; the oracle sums sequentially, and the two agree to
-// rounding.
+// Work decomposition: GB300 issues one FP64 warp instruction per SM in about 19
+// cycles (0.529 T FMA/s measured), so the step is bound by the number of FP64
+// operations per pair and by how evenly they are spread.  What a pair's terms
+// owe to the reference configuration alone (kernel weights, square roots,
+// moduli) is formed once into a table of 32 bytes a pair (ptab), which leaves
+// 12 operations a pair in pass 1 and 53 in pass 2; factors 1 - D_j cost
+// nothing where D_j = 0.  A row is summed by 4 to 16 lanes (with_lanes), so
+// that a small specimen still fills the SMs; the per-particle parts run on
+// consecutive threads.  Forming the terms in place with a warp of 32 rows in
+// series took 10.2 ms per step on 256,000 particles and 0.69 ms on 2048; this
+// form takes 4.1 ms and 0.080 ms.
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tlsph_device.cuh"
 #include "tlsph_internal.cuh"
@@ -65,51 +70,139 @@ __device__ __forceinline__ void apply_bc(const DevState &s, int64_t i, int fail,
     }
 }
 
+// ------------------------------------------------------------------ pair gathers
+// A row is summed by G lanes of a warp that stride over its neighbours; a
+// block of 128 threads holds 128 / G rows, leaves their sums in shared memory
+// and runs the per-particle part with its first 128 / G threads.
+
+// 1 / x: the hardware's first approximation (about 20 bits) refined by one
+// step of Householder's third-order iteration for the reciprocal,
+// r (1 + e + e^2) with e = 1 - x r, whose error e^3 is below FP64 rounding
+__device__ __forceinline__ double rcp_fp64(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// Reference-configuration terms of a pair (kernel normalisations left to the
+// per-row factors): g = V_j W'/r X_ij and, with HG, k = (E_i + E_j) V_j W / X_ij^2.
+// Every rounding is written out, so that a pair's terms read from the table
+// and formed in place are the same bits.
+template <bool HG>
+__device__ __forceinline__ void pair_terms(double dx, double dy, double dz, double inv_h, double Vj, double EE,
+                                           double &gx, double &gy, double &gz, double &k)
+{
+    const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+    const double rinv = rsqrt(r2);
+    const double q = __dmul_rn(__dmul_rn(r2, rinv), inv_h), t = __dsub_rn(2.0, q);
+    double dw = 0.0;
+    if (q < 1.0) dw = __dmul_rn(q, __fma_rn(2.25, q, -3.0));
+    else if (q < 2.0) dw = __dmul_rn(__dmul_rn(-0.75, t), t);
+    const double g = __dmul_rn(__dmul_rn(Vj, dw), rinv);
+    gx = __dmul_rn(g, dx); gy = __dmul_rn(g, dy); gz = __dmul_rn(g, dz);
+    if (HG) {
+        double w = 0.0;
+        if (q < 1.0) w = __fma_rn(-__dmul_rn(q, q), __fma_rn(-0.75, q, 1.5), 1.0);
+        else if (q < 2.0) w = __dmul_rn(__dmul_rn(__dmul_rn(0.25, t), t), t);
+        k = __dmul_rn(__dmul_rn(__dmul_rn(EE, Vj), w), __dmul_rn(rinv, rinv));
+    }
+}
+
+// sum over the G lanes of a row (every lane of the warp takes part)
+template <int G>
+__device__ __forceinline__ double row_sum(double x)
+{
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// The pair table (DevState::ptab, CSR order) and S0_i = sum_j g_ij, summed as
+// pass 2 sums it without the table
+template <int G>
+__global__ void __launch_bounds__(STEP_THREADS) k_pair_table(DevState s, double inv_h, double4_32a *tab, double *S0)
+{
+    const int sub = threadIdx.x % G;
+    const int64_t i = ((int64_t)blockIdx.x * STEP_THREADS + threadIdx.x) / G;
+    double a[3] = { 0.0, 0.0, 0.0 };
+    if (i < s.N) {
+        const double xi = s.X[3 * i], yi = s.X[3 * i + 1], zi = s.X[3 * i + 2], Ei = s.youngs[i];
+        for (int64_t p = s.row_ptr[i] + sub; p < s.row_ptr[i + 1]; p += G) {
+            const int64_t j = s.col[p];
+            double gx, gy, gz, k;
+            pair_terms<true>(s.X[3 * j] - xi, s.X[3 * j + 1] - yi, s.X[3 * j + 2] - zi, inv_h, s.vol[j],
+                             Ei + s.youngs[j], gx, gy, gz, k);
+            tab[p] = make_double4_32a(gx, gy, gz, k);
+            a[0] += gx; a[1] += gy; a[2] += gz;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double t = row_sum<G>(a[c]);
+        if (sub == 0 && i < s.N) S0[3 * i + c] = t;
+    }
+}
+
 // ------------------------------------------------------------------ pass 1
+__device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c, int64_t i, const double *keep);
+
+template <int G>
 __global__ void __launch_bounds__(STEP_THREADS) k_pass1_fp64(DevState s, StepConst c)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) << 5;
-    if (row0 >= s.N) return;
-    const int nrows = (int)min((int64_t)32, s.N - row0);
+    constexpr int ROWS = STEP_THREADS / G;
+    __shared__ double sums[9][ROWS];
+    const int sub = threadIdx.x % G, slot = threadIdx.x / G;
+    const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+    const int64_t i = row0 + slot;
     const double *__restrict__ Dn = s.D[c.dcur];
     const double *__restrict__ X = s.X;
     const double *__restrict__ vh = s.vh;
-    const double *__restrict__ vol = s.vol;
-    double keep[9];
+    const bool tab = s.ptab != nullptr;
+    double m[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) keep[k] = 0.0;
-
-    for (int r = 0; r < nrows; ++r) {
-        const int64_t i = row0 + r;
-        const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
+    for (int k = 0; k < 9; ++k) m[k] = 0.0;
+    if (i < s.N) {
         const double ui = vh[3 * i], vi = vh[3 * i + 1], wi = vh[3 * i + 2];
-        const int64_t p0 = s.row_ptr[i], p1 = s.row_ptr[i + 1];
-        double m[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) m[k] = 0.0;
-        for (int64_t p = p0 + lane; p < p1; p += 32) {
+        const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
+        const int64_t p1 = s.row_ptr[i + 1];
+        for (int64_t p = s.row_ptr[i] + sub; p < p1; p += G) {
             const int64_t j = s.col[p];
-            const double dx = X[3 * j] - xi, dy = X[3 * j + 1] - yi, dz = X[3 * j + 2] - zi;
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double rinv = rsqrt(r2);
-            const double q = r2 * rinv * c.inv_h;
-            const double cw = vol[j] * (1.0 - Dn[j]) * spline_dw(q) * rinv;
-            const double cx = cw * (vh[3 * j] - ui), cy = cw * (vh[3 * j + 1] - vi), cz = cw * (vh[3 * j + 2] - wi);
-            m[0] += cx * dx; m[1] += cx * dy; m[2] += cx * dz;
-            m[3] += cy * dx; m[4] += cy * dy; m[5] += cy * dz;
-            m[6] += cz * dx; m[7] += cz * dy; m[8] += cz * dz;
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const double t = warp_allsum(m[k]);
-            keep[k] = (lane == r) ? t : keep[k];
+            const double Dj = Dn[j];
+            double gx, gy, gz, k;
+            if (tab) {
+                const double4_32a t = s.ptab[p];
+                gx = t.x; gy = t.y; gz = t.z;
+            } else {
+                pair_terms<false>(X[3 * j] - xi, X[3 * j + 1] - yi, X[3 * j + 2] - zi, c.inv_h, s.vol[j], 0.0, gx, gy,
+                                  gz, k);
+            }
+            if (Dj != 0.0) {        // (1 - D_j) g_ij, only where there is damage
+                gx -= Dj * gx; gy -= Dj * gy; gz -= Dj * gz;
+            }
+            const double cx = vh[3 * j] - ui, cy = vh[3 * j + 1] - vi, cz = vh[3 * j + 2] - wi;
+            m[0] += cx * gx; m[1] += cx * gy; m[2] += cx * gz;
+            m[3] += cy * gx; m[4] += cy * gy; m[5] += cy * gz;
+            m[6] += cz * gx; m[7] += cz * gy; m[8] += cz * gz;
         }
     }
-    if (lane >= nrows) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const double t = row_sum<G>(m[k]);
+        if (sub == 0) sums[k][slot] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = sums[k][threadIdx.x];
+    epi1_fp64(s, c, row0 + threadIdx.x, m);
+}
 
-    // ---- per-particle epilogue (one particle per lane)
-    const int64_t i = row0 + lane;
+// per-particle part of pass 1 from the nine sums M (keep)
+__device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c, int64_t i, const double *keep)
+{
+    const double *__restrict__ Dn = s.D[c.dcur];
     double *__restrict__ Dnext = s.D[c.dcur ^ 1];
     const int fail = s.fail[i];
     if (fail >= 0) {            // fully damaged: no stress, F frozen (Sec. 3.1)
@@ -216,93 +309,104 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass1_fp64(DevState s, StepCon
 }
 
 // ------------------------------------------------------------------ pass 2
-template <bool HG>
+__device__ __forceinline__ void epi2_fp64(const DevState &s, const StepConst &c, int64_t i, const double *keep, bool hg);
+
+// sums of row i: 0..2 -sum_j D_j g_ij (the A_i term's part beyond S0_i), 3..5 sum_j A_j g_ij, 6..8 hourglass,
+// 9..11 S0_i where there is no table to hold it
+template <int G, bool HG>
 __global__ void __launch_bounds__(STEP_THREADS) k_pass2_fp64(DevState s, StepConst c)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) << 5;
-    if (row0 >= s.N) return;
-    const int nrows = (int)min((int64_t)32, s.N - row0);
+    constexpr int ROWS = STEP_THREADS / G;
+    __shared__ double sums[12][ROWS];
+    const int sub = threadIdx.x % G, slot = threadIdx.x / G;
+    const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+    const int64_t i = row0 + slot;
     const double *__restrict__ D1 = s.D[c.dcur ^ 1];
     const double *__restrict__ X = s.X;
     const double *__restrict__ un = s.u[c.ucur ^ 1];   // u^{n+1}
-    const double *__restrict__ vol = s.vol;
     const double *__restrict__ Aa = s.A;
     const double *__restrict__ Fa = s.F;
-    double keep[9];
+    const bool tab = s.ptab != nullptr;
+    double acc[12];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) keep[k] = 0.0;
-
-    for (int r = 0; r < nrows; ++r) {
-        const int64_t i = row0 + r;
+    for (int k = 0; k < 12; ++k) acc[k] = 0.0;
+    if (i < s.N) {
         const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
-        double uxi = 0, uyi = 0, uzi = 0, Ei = 0;
-        double Fi[9];
+        double u2x = 0.0, u2y = 0.0, u2z = 0.0, Ei = 0.0;
+        double Hi[9];                       // F_i - 2 I, so that F_j + H_i = (F_i - I) + (F_j - I)
         if (HG) {
-            uxi = un[3 * i]; uyi = un[3 * i + 1]; uzi = un[3 * i + 2];
+            u2x = 2.0 * un[3 * i]; u2y = 2.0 * un[3 * i + 1]; u2z = 2.0 * un[3 * i + 2];
             Ei = s.youngs[i];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) Fi[k] = Fa[9 * i + k];
+            for (int k = 0; k < 9; ++k) Hi[k] = Fa[9 * i + k] - ((k & 3) == 0 ? 2.0 : 0.0);
         }
-        const int64_t p0 = s.row_ptr[i], p1 = s.row_ptr[i + 1];
-        double acc[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-        for (int64_t p = p0 + lane; p < p1; p += 32) {
+        const int64_t p1 = s.row_ptr[i + 1];
+        for (int64_t p = s.row_ptr[i] + sub; p < p1; p += G) {
             const int64_t j = s.col[p];
+            const double Dj = D1[j];
             const double dx = X[3 * j] - xi, dy = X[3 * j + 1] - yi, dz = X[3 * j + 2] - zi;
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double rinv = rsqrt(r2);
-            const double q = r2 * rinv * c.inv_h;
-            const double Vj = vol[j];
-            const double omd = 1.0 - D1[j];
-            const double g = spline_dw(q) * rinv;
-            // s1 = sum V_j (1 - D_j) grad W ; s2 = sum V_j A_j grad W
-            const double c1 = Vj * omd * g;
-            acc[0] += c1 * dx; acc[1] += c1 * dy; acc[2] += c1 * dz;
+            double gx, gy, gz, kh = 0.0;
+            if (tab) {
+                const double4_32a t = s.ptab[p];
+                gx = t.x; gy = t.y; gz = t.z; kh = t.w;
+            } else {
+                pair_terms<HG>(dx, dy, dz, c.inv_h, s.vol[j], HG ? Ei + s.youngs[j] : 0.0, gx, gy, gz, kh);
+                acc[9] += gx; acc[10] += gy; acc[11] += gz;
+            }
             const double *Aj = Aa + 9 * j;
-            const double c2 = Vj * g;
-            acc[3] += c2 * (Aj[0] * dx + Aj[1] * dy + Aj[2] * dz);
-            acc[4] += c2 * (Aj[3] * dx + Aj[4] * dy + Aj[5] * dz);
-            acc[5] += c2 * (Aj[6] * dx + Aj[7] * dy + Aj[8] * dz);
+            acc[3] += Aj[0] * gx; acc[3] += Aj[1] * gy; acc[3] += Aj[2] * gz;
+            acc[4] += Aj[3] * gx; acc[4] += Aj[4] * gy; acc[4] += Aj[5] * gz;
+            acc[5] += Aj[6] * gx; acc[5] += Aj[7] * gy; acc[5] += Aj[8] * gz;
+            if (Dj != 0.0) {
+                acc[0] -= Dj * gx; acc[1] -= Dj * gy; acc[2] -= Dj * gz;
+                if (HG) kh -= Dj * kh;
+            }
             if (HG) {
-                const double xx = dx + un[3 * j] - uxi, xy = dy + un[3 * j + 1] - uyi, xz = dz + un[3 * j + 2] - uzi;
+                // e = ((F_i - I) + (F_j - I)) X_ij - 2 u_ij is eps_i + eps_j; x_ij = X_ij + u_ij;
+                // the force runs along x_ij: k (e . x) / |x|^2 x, with the 1/2 of the pair modulus in the epilogue
+                const double *Fj = Fa + 9 * j;
+                double ex = fma(-2.0, un[3 * j], u2x), ey = fma(-2.0, un[3 * j + 1], u2y), ez = fma(-2.0, un[3 * j + 2], u2z);
+                const double xx = fma(-0.5, ex, dx), xy = fma(-0.5, ey, dy), xz = fma(-0.5, ez, dz);
+                ex += (Hi[0] + Fj[0]) * dx; ex += (Hi[1] + Fj[1]) * dy; ex += (Hi[2] + Fj[2]) * dz;
+                ey += (Hi[3] + Fj[3]) * dx; ey += (Hi[4] + Fj[4]) * dy; ey += (Hi[5] + Fj[5]) * dz;
+                ez += (Hi[6] + Fj[6]) * dx; ez += (Hi[7] + Fj[7]) * dy; ez += (Hi[8] + Fj[8]) * dz;
                 const double lx2 = xx * xx + xy * xy + xz * xz;
-                if (lx2 > 0.0) {
-                    const double lxi = rsqrt(lx2);
-                    const double *Fj = Fa + 9 * j;
-                    const double gx = (Fi[0] + Fj[0]) * dx + (Fi[1] + Fj[1]) * dy + (Fi[2] + Fj[2]) * dz;
-                    const double gy = (Fi[3] + Fj[3]) * dx + (Fi[4] + Fj[4]) * dy + (Fi[5] + Fj[5]) * dz;
-                    const double gz = (Fi[6] + Fj[6]) * dx + (Fi[7] + Fj[7]) * dy + (Fi[8] + Fj[8]) * dz;
-                    // delta = (eps_i + eps_j) . xhat = ((F_i + F_j) X_ij) . xhat - 2 |x_ij|
-                    const double delta = (gx * xx + gy * xy + gz * xz) * lxi - 2.0 * lx2 * lxi;
-                    // pair modulus (E_i + E_j) / 2; the 1/2 is in the epilogue's coefficient
-                    const double ch = (Ei + s.youngs[j]) * omd * Vj * spline_w(q) * rinv * rinv * delta * lxi;
-                    acc[6] += ch * xx; acc[7] += ch * xy; acc[8] += ch * xz;
-                }
+                double ch = kh * (ex * xx + ey * xy + ez * xz) * rcp_fp64(lx2);
+                if (__double2hiint(lx2) < 0x00100000) ch = 0.0;     // coincident current positions: no direction
+                acc[6] += ch * xx; acc[7] += ch * xy; acc[8] += ch * xz;
             }
         }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            if (!HG && k >= 6) continue;
-            const double t = warp_allsum(acc[k]);
-            keep[k] = (lane == r) ? t : keep[k];
-        }
     }
-    if (lane >= nrows) return;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        if ((!HG && k >= 6 && k < 9) || (k >= 9 && tab)) continue;
+        const double t = row_sum<G>(acc[k]);
+        if (sub == 0) sums[k][slot] = t;
+    }
+    __syncthreads();
+    const int64_t r = row0 + threadIdx.x;
+    if (threadIdx.x >= ROWS || r >= s.N) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k] = HG || k < 6 ? sums[k][threadIdx.x] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k] += tab ? s.ps0[3 * r + k] : sums[9 + k][threadIdx.x];
+    epi2_fp64(s, c, r, acc, HG);
+}
 
-    // ---- epilogue: nodal force and velocity-Verlet update of particle i
-    const int64_t i = row0 + lane;
-    const double Vi = vol[i];
-    const double omdi = 1.0 - D1[i];
+// nodal force and velocity-Verlet update of particle i from its sums
+__device__ __forceinline__ void epi2_fp64(const DevState &s, const StepConst &c, int64_t i, const double *keep, bool hg)
+{
+    const double *__restrict__ un = s.u[c.ucur ^ 1];
+    const double Vi = s.vol[i];
+    const double omdi = 1.0 - s.D[c.dcur ^ 1][i];
     double Ai[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Ai[k] = Aa[9 * i + k];
+    for (int k = 0; k < 9; ++k) Ai[k] = s.A[9 * i + k];
     double f[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         f[k] = Vi * c.dw_norm * (Ai[3 * k] * keep[0] + Ai[3 * k + 1] * keep[1] + Ai[3 * k + 2] * keep[2] + omdi * keep[3 + k]);
-    if (HG) {
+    if (hg) {
         const double hc = 0.5 * c.hg_coef * omdi * Vi * c.w_norm;
 #pragma unroll
         for (int k = 0; k < 3; ++k) f[k] += hc * keep[6 + k];
@@ -662,19 +766,43 @@ cudaError_t launch_predict(const DevState &s, int ucur, double dt, bool wall, in
     return cudaGetLastError();
 }
 
+// Lanes per row.  Few lanes waste least (idle lanes of a row's last pairs, row
+// sums, a per-particle part that fills its warps), many lanes spread a small
+// specimen over more warps.  Measured, ms per step with 4 / 8 / 16 lanes:
+// 2048 particles 0.127 / 0.087 / 0.080, 5148 0.158 / 0.140 / 0.163, 12,000 0.253 / 0.270 / 0.297,
+// 42,693 0.791 / 0.860 / 1.057, 256,000 4.08 / 4.57 / 5.86.
+template <class F>
+static void with_lanes(int64_t N, F &&f)
+{
+    if (N < 4096) f(std::integral_constant<int, 16>());
+    else if (N < 8192) f(std::integral_constant<int, 8>());
+    else f(std::integral_constant<int, 4>());
+}
+
 cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucur, int dcur,
                              int64_t step_index, cudaStream_t st, cudaEvent_t *ev)
 {
     const StepConst c = make_const(cfg, ucur, dcur, step_index);
-    const unsigned grid = nblk((s.N + 31) / 32 * 32, STEP_THREADS);
     if (ev) cudaEventRecord(ev[0], st);
-    k_pass1_fp64<<<grid, STEP_THREADS, 0, st>>>(s, c);
-    if (ev) cudaEventRecord(ev[1], st);
-    if (cfg.hg_alpha != 0.0)
-        k_pass2_fp64<true><<<grid, STEP_THREADS, 0, st>>>(s, c);
-    else
-        k_pass2_fp64<false><<<grid, STEP_THREADS, 0, st>>>(s, c);
+    const auto run = [&](auto lanes) {
+        constexpr int G = decltype(lanes)::value;
+        const unsigned grid = nblk(s.N, STEP_THREADS / G);
+        k_pass1_fp64<G><<<grid, STEP_THREADS, 0, st>>>(s, c);
+        if (ev) cudaEventRecord(ev[1], st);
+        if (cfg.hg_alpha != 0.0) k_pass2_fp64<G, true><<<grid, STEP_THREADS, 0, st>>>(s, c);
+        else k_pass2_fp64<G, false><<<grid, STEP_THREADS, 0, st>>>(s, c);
+    };
+    with_lanes(s.N, run);
     if (ev) cudaEventRecord(ev[2], st);
+    return cudaGetLastError();
+}
+
+cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, cudaStream_t st)
+{
+    with_lanes(s.N, [&](auto lanes) {
+        constexpr int G = decltype(lanes)::value;
+        k_pair_table<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, 1.0 / h, tab, S0);
+    });
     return cudaGetLastError();
 }
 

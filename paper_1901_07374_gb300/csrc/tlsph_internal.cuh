@@ -95,6 +95,10 @@ struct DevState {
     FixPack pack;
     double grip_ramp = 0.0;  // tau of the grip velocity ramp (Sec. 6); 0: constant prescribed velocities
     double *e = nullptr;     // N   specific internal energy (Eq. conservation3)
+    // FP64 path: reference-configuration terms of every pair in CSR order,
+    // {g = V_j W'/r X_ij, k = (E_i + E_j) V_j W / X_ij^2}, and S0_i = sum_j g_ij (null: formed in place)
+    const double4_32a *ptab = nullptr;  // nnz
+    const double *ps0 = nullptr;    // N*3
 };
 
 // The pass-2 record is tiled by 32 particles: component k (0..5) of particle j
@@ -152,6 +156,7 @@ struct tlsph_ctx {
     void *w1t_mem = nullptr;    // library-owned pass-1 weight table (pass-1 plan form 5) and its offsets
     void *w1t_off_mem = nullptr;
     void *col_mem = nullptr;    // library-owned CSR columns
+    void *ptab_mem = nullptr;   // library-owned pair table of the FP64 path, its S0 behind it
     int32_t *perm_dev = nullptr;
     int32_t *inv_dev = nullptr;   // device copy of inv when reordered, else null (identity)
     std::vector<int32_t> perm, inv;   // host copies of the order when reordered (empty in caller order)
@@ -224,6 +229,7 @@ __host__ __device__ inline void wall_contact(double Xz, double &uz, double &vz)
 // ev: null, or 3 events recorded before pass 1, between the passes and after pass 2
 cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucur, int dcur,
                              int64_t step_index, cudaStream_t st, cudaEvent_t *ev);
+cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, cudaStream_t st);
 cudaError_t launch_material_point_value(const DevMat &m, double dt, int64_t n, const double *deps,
                                         const double *J, double *state, cudaStream_t st);
 cudaError_t launch_export_sym(const double *src6, double *dst9, int64_t N, cudaStream_t st);
