@@ -414,17 +414,6 @@ __device__ __forceinline__ void df_split(double x, float &h, float &l)
 }
 __device__ __forceinline__ double df_value(float h, float l) { return (double)h + (double)l; }
 
-// single-precision flow stress sigma_f of Algorithm 1 (Johnson-Cook hardening
-// and lagged rate factor, as jc_hard * jc_rate)
-__device__ __forceinline__ float jc_flow_f(const DevMat &m, float ep, float epdot)
-{
-    float r = 1.0f;
-    if (m.Cf != 0.0f && m.inv_epsdot0f > 0.0f) {
-        const float x = epdot * m.inv_epsdot0f;
-        if (x > 1.0f) r = 1.0f + m.Cf * logf(x);
-    }
-    return (ep > 0.0f ? m.Af + m.Bf * powf(ep, m.nf) : m.Af) * r;
-}
 // single-precision mean stress (eos_sm) from J - 1
 __device__ __forceinline__ float eos_sm_f(const DevMat &m, float Jm1, float J, float D, float e)
 {

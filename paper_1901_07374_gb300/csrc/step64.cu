@@ -75,17 +75,6 @@ __device__ __forceinline__ void apply_bc(const DevState &s, int64_t i, int fail,
 // block of 128 threads holds 128 / G rows, leaves their sums in shared memory
 // and runs the per-particle part with its first 128 / G threads.
 
-// 1 / x: the hardware's first approximation (about 20 bits) refined by one
-// step of Householder's third-order iteration for the reciprocal,
-// r (1 + e + e^2) with e = 1 - x r, whose error e^3 is below FP64 rounding
-__device__ __forceinline__ double rcp_fp64(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // Reference-configuration terms of a pair (kernel normalisations left to the
 // per-row factors): g = V_j W'/r X_ij and, with HG, k = (E_i + E_j) V_j W / X_ij^2.
 // Every rounding is written out, so that a pair's terms read from the table
@@ -231,7 +220,7 @@ __device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c,
         return;
     }
     // F^{-1} = cof^T / J ;  L_v = Fdot F^{-1} ;  d = sym(L_v)
-    const double iJ = 1.0 / J;
+    const double iJ = rcp_fp64(J);
     double Fi[9];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -241,7 +230,7 @@ __device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c,
     mul3(Fd, Fi, Lv);
     const double d[6] = { Lv[0], Lv[4], Lv[8], 0.5 * (Lv[1] + Lv[3]), 0.5 * (Lv[5] + Lv[7]), 0.5 * (Lv[2] + Lv[6]) };
     double R[9];
-    uint32_t st = polar_rotation(Fn, R) ? 0u : TLSPH_ST_POLAR_CAP;
+    uint32_t st = polar_rotation(Fn, Fi, R) ? 0u : TLSPH_ST_POLAR_CAP;
     double dh[6];
     sym_rotate_t(R, d, dh);
     double de[6];
@@ -260,7 +249,7 @@ __device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c,
     mp.e = s.e[i];
     mp.failed = 0;
     const DevMat &mat = s.mats[s.mat[i]];
-    st |= material_update(mat, c.dt, de, J, mp);
+    st |= material_update<false, true>(mat, c.dt, de, J, mp);
     // internal energy (Eq. conservation3, de/dt = J sigma : d / rho0), trapezoidal in the step with the
     // stress at its start and at its end (zero after a failure), current frame, d scaled by dt below
     double sgn[6];

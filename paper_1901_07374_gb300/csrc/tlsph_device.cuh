@@ -152,35 +152,59 @@ __device__ __forceinline__ void sym_rotate(const double *Q, const double *s, dou
 #undef QT
 }
 
+// 1 / x: the hardware's first approximation (about 20 bits) refined by one
+// step of Householder's third-order iteration for the reciprocal,
+// r (1 + e + e^2) with e = 1 - x r, whose error e^3 is below FP64 rounding
+__device__ __forceinline__ double rcp_fp64(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 // Rotation factor of the polar decomposition F = R U by Newton's iteration
 // X <- (g X + X^{-T} / g) / 2 with the determinant scaling g = |det X|^{-1/3}
-// (N. J. Higham, "Computing the polar decomposition -- with applications",
-// SIAM J. Sci. Stat. Comput. 7, 1986).  Converges quadratically; the loop
-// stops once a step moves X by less than 1e-10 (the next iterate is then
-// exact to rounding) and is capped at 30 steps (status bit on the cap).
-__device__ __forceinline__ bool polar_rotation(const double *F, double *R)
+// while X is far from a rotation and g = 1 near it (N. J. Higham, "Computing
+// the polar decomposition -- with applications", SIAM J. Sci. Stat. Comput. 7,
+// 1986).  FiT = F^{-T} is the first step's inverse, which the caller has.  A
+// step that moves no entry by 2^-28 leaves an error below its square, under
+// FP64 rounding: that iterate is the result.  Three steps (about 150 FP64
+// operations) at strains of a percent.  Capped at 32 steps (status bit on the
+// cap).  The move is compared by the entries' exponent words, on the integer
+// pipe.
+__device__ __forceinline__ bool polar_rotation(const double *F, const double *Fi, double *R)
 {
+    int move = 0;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) R[k] = F[k];
-    bool last = false;
-    for (int it = 0; it < 30; ++it) {
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const double x = 0.5 * (F[3 * k + l] + Fi[3 * l + k]);
+            move = max(move, __double2hiint(x - F[3 * k + l]) & 0x7fffffff);
+            R[3 * k + l] = x;
+        }
+    for (int it = 1; it < 32; ++it) {
+        if (move < 0x3e300000) return true;             // every entry moved by less than 2^-28
+        const bool far = move >= 0x3fc00000;             // an entry moved by 2^-3 or more
         double c[9];
         cof3(R, c);
-        double d = R[0] * c[0] + R[1] * c[1] + R[2] * c[2];
-        double g = rcbrt(fabs(d));
-        double ginv_d = 1.0 / (g * d);
-        double diff = 0.0;
+        const double d = R[0] * c[0] + R[1] * c[1] + R[2] * c[2];
+        double h = 0.5, q = 0.5 * rcp_fp64(d);
+        if (far) {
+            const double g = rcbrt(fabs(d));
+            h = 0.5 * g;
+            q = 0.5 / (g * d);
+        }
+        move = 0;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            double xn = 0.5 * (g * R[k] + c[k] * ginv_d);
-            double e = xn - R[k];
-            diff += e * e;
-            R[k] = xn;
+            const double x = fma(q, c[k], h * R[k]);
+            move = max(move, __double2hiint(x - R[k]) & 0x7fffffff);
+            R[k] = x;
         }
-        if (last) return true;
-        if (diff < 1e-20) last = true;
     }
-    return false;
+    return move < 0x3e300000;
 }
 
 // Largest eigenvalue of a symmetric 3x3 (6) by the trigonometric solution of
@@ -413,10 +437,26 @@ __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const d
     return de;
 }
 
+// Single-precision flow stress sigma_f / (1 - D) of Algorithm 1 (Johnson-Cook
+// hardening and lagged rate factor, as jc_hard * jc_rate)
+__device__ __forceinline__ float jc_flow_f(const DevMat &m, float ep, float epdot)
+{
+    float r = 1.0f;
+    if (m.Cf != 0.0f && m.inv_epsdot0f > 0.0f) {
+        const float x = epdot * m.inv_epsdot0f;
+        if (x > 1.0f) r = 1.0f + m.Cf * logf(x);
+    }
+    return (ep > 0.0f ? m.Af + m.Bf * powf(ep, m.nf) : m.Af) * r;
+}
+
 // Constitutive and damage update of one particle from the symmetric strain
 // increment de (unrotated frame) and J = det F^{n+1}.  D^n enters, D^{n+1}
-// leaves.  Returns status bits.
-template <bool SEED32 = false>
+// leaves.  Returns status bits.  SCREEN spares a particle well inside its
+// yield surface the FP64 power and logarithm of the flow stress: FP32 values
+// of sigma_eq^2 and sigma_f^2 are within 2e-6 of the FP64 ones, so
+// sigma_eq^2 <= sigma_f^2 (1 - 1e-5) in FP32 implies the FP64 test, and the
+// elastic branch does not use sigma_f.
+template <bool SEED32 = false, bool SCREEN = false>
 __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, const double *de, double J,
                                                     MPState &s)
 {
@@ -434,9 +474,18 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
 #pragma unroll
         for (int k = 0; k < 6; ++k) tr[k] = s.sd[k] + 2.0 * m.G * omD * ed[k];
         const double s2 = 1.5 * sym_ddot(tr, tr);
-        const double sf = jc_hard(m, s.ep) * jc_rate(m, s.epdot) * omD;
+        double sf = 0.0;
+        bool elastic = false;
+        if (SCREEN && s.ep > 0.0) {
+            const float f = jc_flow_f(m, (float)s.ep, (float)s.epdot) * (float)omD;
+            elastic = f > 0.0f && (float)s2 <= f * f * (1.0f - 1e-5f);
+        }
+        if (!elastic) {
+            sf = jc_hard(m, s.ep) * jc_rate(m, s.epdot) * omD;
+            elastic = s2 <= sf * sf;    // sigma_eq <= sigma_f, decided without the square root
+        }
         dep = 0.0;
-        if (s2 <= sf * sf) {            // sigma_eq <= sigma_f, decided without the square root
+        if (elastic) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) s.sd[k] = tr[k];
         } else {
