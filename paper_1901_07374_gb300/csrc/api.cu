@@ -387,7 +387,8 @@ DevMat make_dev_mat(const tlsph_material &m)
 
 // The pair table of an FP64 context in library-owned memory, formed once every
 // material it uses is set and again when one is set anew (its entries hold
-// Young's moduli).  32 bytes a pair: 0.8 GB for 256,000 particles.  It is left
+// Young's moduli).  52 bytes a pair with the pair numbers and the hourglass
+// vectors: 1.3 GB for 256,000 particles.  It is left
 // out (the steps then form the terms in place) where it would take more than a
 // quarter of the free device memory, so that it never decides how many
 // contexts fit.
@@ -396,21 +397,30 @@ static cudaError_t ctx_pair_table(tlsph_ctx *ctx)
     if (ctx->cfg.precision != TLSPH_PRECISION_FP64 || !ctx->owns_mem || ctx->nnz == 0) return cudaSuccess;
     for (int k = 0; k < TLSPH_MAX_MATERIALS; ++k)
         if (ctx->mat_used[k] && !ctx->mat_set[k]) return cudaSuccess;
-    const size_t tab = (size_t)ctx->nnz * sizeof(double4_32a), bytes = tab + 3 * (size_t)ctx->N * sizeof(double);
+    const size_t n = (size_t)ctx->N, nnz = (size_t)ctx->nnz;
+    Carver c;
+    const size_t o_tab = c.take(nnz * sizeof(double4_32a)), o_w = c.take(nnz / 2 * sizeof(double4_32a));
+    const size_t o_id = c.take(nnz * sizeof(int32_t)), o_s0 = c.take(3 * n * sizeof(double));
+    const size_t o_uoff = c.take((n + 1) * sizeof(int64_t)), o_scan = c.take(scan_tmp_elems(ctx->N + 1) * sizeof(int64_t));
     if (!ctx->ptab_mem) {
         size_t avail = 0, total = 0;
-        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || bytes > avail / 4 ||
-            cudaMalloc(&ctx->ptab_mem, bytes) != cudaSuccess) {
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || c.off > avail / 4 ||
+            cudaMalloc(&ctx->ptab_mem, c.off) != cudaSuccess) {
             cudaGetLastError();
             ctx->ptab_mem = nullptr;
             return cudaSuccess;
         }
     }
-    double *S0 = reinterpret_cast<double *>(static_cast<char *>(ctx->ptab_mem) + tab);
-    const cudaError_t e = build_pair_table(ctx->s, ctx->cfg.h, static_cast<double4_32a *>(ctx->ptab_mem), S0, ctx->stream);
+    void *base = ctx->ptab_mem;
+    const cudaError_t e = build_pair_table(ctx->s, ctx->cfg.h, at<double4_32a>(base, o_tab), at<double>(base, o_s0),
+                                           at<int64_t>(base, o_uoff), at<int64_t>(base, o_scan), at<int32_t>(base, o_id),
+                                           ctx->stream);
     if (e != cudaSuccess) return e;
-    ctx->s.ptab = static_cast<const double4_32a *>(ctx->ptab_mem);
-    ctx->s.ps0 = S0;
+    ctx->s.ptab = at<double4_32a>(base, o_tab);
+    ctx->s.pw = at<double4_32a>(base, o_w);
+    ctx->s.pid = at<int32_t>(base, o_id);
+    ctx->s.ps0 = at<double>(base, o_s0);
+    ctx->s.puoff = at<int64_t>(base, o_uoff);
     return cudaSuccess;
 }
 

@@ -12,17 +12,22 @@
 // plus hourglass control, then the velocity-Verlet update with the
 // velocity constraints and the fully damaged particles held at rest.
 //
-// Work decomposition: GB300 issues one FP64 warp instruction per SM in about 19
-// cycles (0.529 T FMA/s measured), so the step is bound by the number of FP64
-// operations per pair and by how evenly they are spread.  What a pair's terms
-// owe to the reference configuration alone (kernel weights, square roots,
-// moduli) is formed once into a table of 32 bytes a pair (ptab), which leaves
-// 12 operations a pair in pass 1 and 53 in pass 2; factors 1 - D_j cost
-// nothing where D_j = 0.  A row is summed by 4 to 16 lanes (with_lanes), so
-// that a small specimen still fills the SMs; the per-particle parts run on
-// consecutive threads.  Forming the terms in place with a warp of 32 rows in
-// series took 10.2 ms per step on 256,000 particles and 0.69 ms on 2048; this
-// form takes 4.1 ms and 0.080 ms.
+// Work decomposition: GB300 issues one FP64 warp instruction per SM in 16
+// cycles, so the step is bound by the number of FP64 instructions it issues and
+// by how evenly they are spread (ncu on 160,000 particles: FP64 pipe 74 % busy
+// in pass 1, 89 % in the hourglass pairs, 90 % in pass 2).
+//  - What a pair's terms owe to the reference configuration alone (kernel
+//    weights, square roots, moduli) is formed once into a table of 32 bytes a
+//    pair (ptab): 12 operations a pair stay in pass 1.
+//  - The hourglass vector of a pair (40 operations) is antisymmetric: it is
+//    formed once per unordered pair (k_pair_hourglass) and read by both rows,
+//    which leaves 12 operations a pair in pass 2.
+//  - Factors 1 - D_j are branched over where D_j = 0.
+//  - A row is summed by 2 to 16 lanes (row_lanes), so that a small specimen
+//    still fills the SMs; the per-particle parts run on consecutive threads.
+// ms per step: forming every term in place with a warp of 32 rows in series
+// 10.2 (256,000 particles) and 0.69 (2048); with the table 4.1 and 0.080; with
+// the hourglass vectors shared and the damage branches 2.6 and 0.070.
 #include <math.h>
 
 #include <algorithm>
@@ -99,6 +104,45 @@ __device__ __forceinline__ void pair_terms(double dx, double dy, double dz, doub
     }
 }
 
+// Hourglass vector w_ij = (e . x_ij) x_ij / |x_ij|^2 of a pair, with
+// e = eps_i + eps_j = ((F_i - I) + (F_j - I)) X_ij - 2 u_ij and
+// x_ij = X_ij + u_ij; u2i = 2 u_i.  hd[k] is the k-th diagonal entry of
+// (F_i - I) + (F_j - I), formed as F_b + (F_a - 2) with a < b.  Every rounding
+// is written out and symmetric in i and j, so w_ji = -w_ij bit for bit and a
+// pair's vector formed once serves both of its rows.
+__device__ __forceinline__ void pair_hourglass(double dx, double dy, double dz, const double *u2i, const double *uj,
+                                               const double *Hi, const double *Fj, const double *hd, double *w)
+{
+    double ex = __fma_rn(-2.0, uj[0], u2i[0]), ey = __fma_rn(-2.0, uj[1], u2i[1]), ez = __fma_rn(-2.0, uj[2], u2i[2]);
+    const double xx = __fma_rn(-0.5, ex, dx), xy = __fma_rn(-0.5, ey, dy), xz = __fma_rn(-0.5, ez, dz);
+    ex = __fma_rn(hd[0], dx, ex);
+    ex = __fma_rn(Hi[1] + Fj[1], dy, ex);
+    ex = __fma_rn(Hi[2] + Fj[2], dz, ex);
+    ey = __fma_rn(Hi[3] + Fj[3], dx, ey);
+    ey = __fma_rn(hd[1], dy, ey);
+    ey = __fma_rn(Hi[5] + Fj[5], dz, ey);
+    ez = __fma_rn(Hi[6] + Fj[6], dx, ez);
+    ez = __fma_rn(Hi[7] + Fj[7], dy, ez);
+    ez = __fma_rn(hd[2], dz, ez);
+    const double lx2 = __fma_rn(xz, xz, __fma_rn(xy, xy, __dmul_rn(xx, xx)));
+    double c = __dmul_rn(__fma_rn(ez, xz, __fma_rn(ey, xy, __dmul_rn(ex, xx))), rcp_fp64(lx2));
+    if (__double2hiint(lx2) < 0x00100000) c = 0.0;      // coincident current positions: no direction
+    w[0] = __dmul_rn(c, xx); w[1] = __dmul_rn(c, xy); w[2] = __dmul_rn(c, xz);
+}
+
+// D != 0 by its upper word, on the integer pipe (an FP64 comparison would
+// occupy the pipe that bounds the gathers; a D below 2^-1022 leaves 1 - D = 1)
+__device__ __forceinline__ bool damaged(double D) { return (__double2hiint(D) & 0x7fffffff) != 0; }
+
+// {(1 - D) gx, (1 - D) gy, (1 - D) gz, (1 - D) k}.  A call, not inlined: a
+// condition around so few instructions is predicated otherwise, and predicated
+// FP64 instructions hold the pipe like executed ones (a third of the pipe's
+// time in pass 2 without any damage)
+__device__ __noinline__ double4_32a damp(double D, double gx, double gy, double gz, double k)
+{
+    return make_double4_32a(__fma_rn(-D, gx, gx), __fma_rn(-D, gy, gy), __fma_rn(-D, gz, gz), __fma_rn(-D, k, k));
+}
+
 // sum over the G lanes of a row (every lane of the warp takes part)
 template <int G>
 __device__ __forceinline__ double row_sum(double x)
@@ -111,11 +155,13 @@ __device__ __forceinline__ double row_sum(double x)
 // The pair table (DevState::ptab, CSR order) and S0_i = sum_j g_ij, summed as
 // pass 2 sums it without the table
 template <int G>
-__global__ void __launch_bounds__(STEP_THREADS) k_pair_table(DevState s, double inv_h, double4_32a *tab, double *S0)
+__global__ void __launch_bounds__(STEP_THREADS) k_pair_table(DevState s, double inv_h, double4_32a *tab, double *S0,
+                                                             int64_t *upper)
 {
     const int sub = threadIdx.x % G;
     const int64_t i = ((int64_t)blockIdx.x * STEP_THREADS + threadIdx.x) / G;
     double a[3] = { 0.0, 0.0, 0.0 };
+    int up = 0;
     if (i < s.N) {
         const double xi = s.X[3 * i], yi = s.X[3 * i + 1], zi = s.X[3 * i + 2], Ei = s.youngs[i];
         for (int64_t p = s.row_ptr[i] + sub; p < s.row_ptr[i + 1]; p += G) {
@@ -125,12 +171,66 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pair_table(DevState s, double 
                              Ei + s.youngs[j], gx, gy, gz, k);
             tab[p] = make_double4_32a(gx, gy, gz, k);
             a[0] += gx; a[1] += gy; a[2] += gz;
+            up += j > i;
         }
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const double t = row_sum<G>(a[c]);
         if (sub == 0 && i < s.N) S0[3 * i + c] = t;
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) up += __shfl_xor_sync(0xffffffffu, up, o);
+    if (sub == 0 && i < s.N) upper[i] = up;
+}
+
+// Number of the unordered pair behind every CSR entry: the pairs (i, j > i) of
+// row i are uoff[i], uoff[i] + 1, ... in the order of the row's tail; an entry
+// with j < i finds i in row j's tail by bisection (rows ascend)
+__global__ void __launch_bounds__(STEP_THREADS) k_pair_id(DevState s, const int64_t *uoff, int32_t *id)
+{
+    const int64_t i = ((int64_t)blockIdx.x * STEP_THREADS + threadIdx.x) / 4;
+    if (i >= s.N) return;
+    const int64_t end = s.row_ptr[i + 1], tail = end - (uoff[i + 1] - uoff[i]);
+    for (int64_t p = s.row_ptr[i] + threadIdx.x % 4; p < end; p += 4) {
+        const int64_t j = s.col[p];
+        if (j > i) {
+            id[p] = (int32_t)(uoff[i] + (p - tail));
+            continue;
+        }
+        const int64_t jend = s.row_ptr[j + 1], jtail = jend - (uoff[j + 1] - uoff[j]);
+        int64_t lo = jtail, hi = jend - 1;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (s.col[mid] < i) lo = mid + 1;
+            else hi = mid;
+        }
+        id[p] = (int32_t)(uoff[j] + (lo - jtail));
+    }
+}
+
+// hourglass vectors of the unordered pairs (i, j > i)
+template <int G>
+__global__ void __launch_bounds__(STEP_THREADS) k_pair_hourglass(DevState s, int ucur)
+{
+    const int64_t i = ((int64_t)blockIdx.x * STEP_THREADS + threadIdx.x) / G;
+    if (i >= s.N) return;
+    const double *__restrict__ X = s.X;
+    const double *__restrict__ un = s.u[ucur ^ 1];     // u^{n+1}
+    const double *__restrict__ Fa = s.F;
+    const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
+    const double u2[3] = { 2.0 * un[3 * i], 2.0 * un[3 * i + 1], 2.0 * un[3 * i + 2] };
+    double Hi[9];                                      // F_i, its diagonal less 2
+#pragma unroll
+    for (int k = 0; k < 9; ++k) Hi[k] = Fa[9 * i + k] - ((k & 3) == 0 ? 2.0 : 0.0);
+    const int64_t u0 = s.puoff[i], end = s.row_ptr[i + 1], tail = end - (s.puoff[i + 1] - u0);
+    for (int64_t p = tail + threadIdx.x % G; p < end; p += G) {
+        const int64_t j = s.col[p];
+        const double *Fj = Fa + 9 * j;
+        const double hd[3] = { Fj[0] + Hi[0], Fj[4] + Hi[4], Fj[8] + Hi[8] };
+        double w[3];
+        pair_hourglass(X[3 * j] - xi, X[3 * j + 1] - yi, X[3 * j + 2] - zi, u2, un + 3 * j, Hi, Fj, hd, w);
+        s.pw[u0 + (p - tail)] = make_double4_32a(w[0], w[1], w[2], 0.0);
     }
 }
 
@@ -167,8 +267,9 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass1_fp64(DevState s, StepCon
                 pair_terms<false>(X[3 * j] - xi, X[3 * j + 1] - yi, X[3 * j + 2] - zi, c.inv_h, s.vol[j], 0.0, gx, gy,
                                   gz, k);
             }
-            if (Dj != 0.0) {        // (1 - D_j) g_ij, only where there is damage
-                gx -= Dj * gx; gy -= Dj * gy; gz -= Dj * gz;
+            if (damaged(Dj)) {      // (1 - D_j) g_ij, only where there is damage
+                const double4_32a t = damp(Dj, gx, gy, gz, 0.0);
+                gx = t.x; gy = t.y; gz = t.z;
             }
             const double cx = vh[3 * j] - ui, cy = vh[3 * j + 1] - vi, cz = vh[3 * j + 2] - wi;
             m[0] += cx * gx; m[1] += cx * gy; m[2] += cx * gz;
@@ -319,51 +420,62 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass2_fp64(DevState s, StepCon
     double acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = 0.0;
-    if (i < s.N) {
-        const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
-        double u2x = 0.0, u2y = 0.0, u2z = 0.0, Ei = 0.0;
-        double Hi[9];                       // F_i - 2 I, so that F_j + H_i = (F_i - I) + (F_j - I)
-        if (HG) {
-            u2x = 2.0 * un[3 * i]; u2y = 2.0 * un[3 * i + 1]; u2z = 2.0 * un[3 * i + 2];
-            Ei = s.youngs[i];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) Hi[k] = Fa[9 * i + k] - ((k & 3) == 0 ? 2.0 : 0.0);
+    const auto pair = [&](int64_t j, double gx, double gy, double gz, double kh, const double *w) {
+        const double Dj = D1[j];
+        const double *Aj = Aa + 9 * j;
+        acc[3] = __fma_rn(Aj[2], gz, __fma_rn(Aj[1], gy, __fma_rn(Aj[0], gx, acc[3])));
+        acc[4] = __fma_rn(Aj[5], gz, __fma_rn(Aj[4], gy, __fma_rn(Aj[3], gx, acc[4])));
+        acc[5] = __fma_rn(Aj[8], gz, __fma_rn(Aj[7], gy, __fma_rn(Aj[6], gx, acc[5])));
+        if (damaged(Dj)) {
+            const double4_32a t = damp(Dj, gx, gy, gz, kh);
+            acc[0] += t.x - gx;
+            acc[1] += t.y - gy;
+            acc[2] += t.z - gz;
+            kh = t.w;
         }
+        if (HG) {   // the 1/2 of the pair modulus is in the epilogue's coefficient
+            acc[6] = __fma_rn(kh, w[0], acc[6]);
+            acc[7] = __fma_rn(kh, w[1], acc[7]);
+            acc[8] = __fma_rn(kh, w[2], acc[8]);
+        }
+    };
+    if (i < s.N && tab) {
         const int64_t p1 = s.row_ptr[i + 1];
         for (int64_t p = s.row_ptr[i] + sub; p < p1; p += G) {
             const int64_t j = s.col[p];
-            const double Dj = D1[j];
-            const double dx = X[3 * j] - xi, dy = X[3 * j + 1] - yi, dz = X[3 * j + 2] - zi;
-            double gx, gy, gz, kh = 0.0;
-            if (tab) {
-                const double4_32a t = s.ptab[p];
-                gx = t.x; gy = t.y; gz = t.z; kh = t.w;
-            } else {
-                pair_terms<HG>(dx, dy, dz, c.inv_h, s.vol[j], HG ? Ei + s.youngs[j] : 0.0, gx, gy, gz, kh);
-                acc[9] += gx; acc[10] += gy; acc[11] += gz;
-            }
-            const double *Aj = Aa + 9 * j;
-            acc[3] += Aj[0] * gx; acc[3] += Aj[1] * gy; acc[3] += Aj[2] * gz;
-            acc[4] += Aj[3] * gx; acc[4] += Aj[4] * gy; acc[4] += Aj[5] * gz;
-            acc[5] += Aj[6] * gx; acc[5] += Aj[7] * gy; acc[5] += Aj[8] * gz;
-            if (Dj != 0.0) {
-                acc[0] -= Dj * gx; acc[1] -= Dj * gy; acc[2] -= Dj * gz;
-                if (HG) kh -= Dj * kh;
-            }
+            const double4_32a t = s.ptab[p];
+            double w[3] = { 0.0, 0.0, 0.0 }, kh = t.w;
             if (HG) {
-                // e = ((F_i - I) + (F_j - I)) X_ij - 2 u_ij is eps_i + eps_j; x_ij = X_ij + u_ij;
-                // the force runs along x_ij: k (e . x) / |x|^2 x, with the 1/2 of the pair modulus in the epilogue
-                const double *Fj = Fa + 9 * j;
-                double ex = fma(-2.0, un[3 * j], u2x), ey = fma(-2.0, un[3 * j + 1], u2y), ez = fma(-2.0, un[3 * j + 2], u2z);
-                const double xx = fma(-0.5, ex, dx), xy = fma(-0.5, ey, dy), xz = fma(-0.5, ez, dz);
-                ex += (Hi[0] + Fj[0]) * dx; ex += (Hi[1] + Fj[1]) * dy; ex += (Hi[2] + Fj[2]) * dz;
-                ey += (Hi[3] + Fj[3]) * dx; ey += (Hi[4] + Fj[4]) * dy; ey += (Hi[5] + Fj[5]) * dz;
-                ez += (Hi[6] + Fj[6]) * dx; ez += (Hi[7] + Fj[7]) * dy; ez += (Hi[8] + Fj[8]) * dz;
-                const double lx2 = xx * xx + xy * xy + xz * xz;
-                double ch = kh * (ex * xx + ey * xy + ez * xz) * rcp_fp64(lx2);
-                if (__double2hiint(lx2) < 0x00100000) ch = 0.0;     // coincident current positions: no direction
-                acc[6] += ch * xx; acc[7] += ch * xy; acc[8] += ch * xz;
+                const double4_32a v = s.pw[s.pid[p]];
+                w[0] = v.x; w[1] = v.y; w[2] = v.z;
+                // w_ij = -w_ji: the sign is the top bit, set on the integer pipe
+                kh = __longlong_as_double(__double_as_longlong(kh) ^ ((long long)(j < i) << 63));
             }
+            pair(j, t.x, t.y, t.z, kh, w);
+        }
+    } else if (i < s.N) {
+        const double xi = X[3 * i], yi = X[3 * i + 1], zi = X[3 * i + 2];
+        const double Ei = s.youngs[i];
+        double u2[3], Fi[9];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u2[k] = 2.0 * un[3 * i + k];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) Fi[k] = Fa[9 * i + k];
+        const int64_t p1 = s.row_ptr[i + 1];
+        for (int64_t p = s.row_ptr[i] + sub; p < p1; p += G) {
+            const int64_t j = s.col[p];
+            const double dx = X[3 * j] - xi, dy = X[3 * j + 1] - yi, dz = X[3 * j + 2] - zi;
+            double gx, gy, gz, kh = 0.0, w[3] = { 0.0, 0.0, 0.0 };
+            pair_terms<HG>(dx, dy, dz, c.inv_h, s.vol[j], HG ? Ei + s.youngs[j] : 0.0, gx, gy, gz, kh);
+            acc[9] += gx; acc[10] += gy; acc[11] += gz;
+            if (HG) {
+                const double *Fj = Fa + 9 * j;
+                double hd[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) hd[k] = j < i ? Fi[4 * k] + (Fj[4 * k] - 2.0) : Fj[4 * k] + (Fi[4 * k] - 2.0);
+                pair_hourglass(dx, dy, dz, u2, un + 3 * j, Fi, Fj, hd, w);
+            }
+            pair(j, gx, gy, gz, kh, w);
         }
     }
 #pragma unroll
@@ -757,15 +869,24 @@ cudaError_t launch_predict(const DevState &s, int ucur, double dt, bool wall, in
 
 // Lanes per row.  Few lanes waste least (idle lanes of a row's last pairs, row
 // sums, a per-particle part that fills its warps), many lanes spread a small
-// specimen over more warps.  Measured, ms per step with 4 / 8 / 16 lanes:
-// 2048 particles 0.127 / 0.087 / 0.080, 5148 0.158 / 0.140 / 0.163, 12,000 0.253 / 0.270 / 0.297,
-// 42,693 0.791 / 0.860 / 1.057, 256,000 4.08 / 4.57 / 5.86.
+// specimen over more warps.  Measured, ms with 2 / 4 / 8 / 16 lanes:
+//   particles    pass 1                     hourglass pairs            pass 2
+//   2048         .064 / .047 / .038 / .035  .054 / .031 / .019 / .018  .049 / .030 / .021 / .017
+//   5148         .069 / .049 / .043 / .064  .056 / .042 / .037 / .036  .054 / .033 / .027 / .038
+//   12,000       .086 / .067 / .075 / .108  .089 / .068 / .063 / .067  .056 / .043 / .057 / .059
+//   42,693       .211 / .206 / .272 / .383  .217 / .202 / .205 / .237  .163 / .142 / .151 / .186
+//   256,000      .878 / 1.00 / 1.36 / 2.18  1.10 / 1.10 / 1.16 / 1.41  .658 / .664 / .789 / 1.05
+static int row_lanes(int64_t N) { return N < 4096 ? 16 : (N < 8192 ? 8 : 4); }                      // pass 2, pair table
+static int pass1_lanes(int64_t N) { return N >= 100000 ? 2 : row_lanes(N); }
+static int hourglass_lanes(int64_t N) { return N < 8192 ? 16 : (N < 32768 ? 8 : 4); }
+
 template <class F>
-static void with_lanes(int64_t N, F &&f)
+static void with_lanes(int lanes, F &&f)
 {
-    if (N < 4096) f(std::integral_constant<int, 16>());
-    else if (N < 8192) f(std::integral_constant<int, 8>());
-    else f(std::integral_constant<int, 4>());
+    if (lanes == 2) f(std::integral_constant<int, 2>());
+    else if (lanes == 4) f(std::integral_constant<int, 4>());
+    else if (lanes == 8) f(std::integral_constant<int, 8>());
+    else f(std::integral_constant<int, 16>());
 }
 
 cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucur, int dcur,
@@ -773,25 +894,39 @@ cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucu
 {
     const StepConst c = make_const(cfg, ucur, dcur, step_index);
     if (ev) cudaEventRecord(ev[0], st);
-    const auto run = [&](auto lanes) {
+    with_lanes(pass1_lanes(s.N), [&](auto lanes) {
+        constexpr int G = decltype(lanes)::value;
+        k_pass1_fp64<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, c);
+    });
+    if (ev) cudaEventRecord(ev[1], st);
+    const bool hg = cfg.hg_alpha != 0.0;
+    if (hg && s.ptab)
+        with_lanes(hourglass_lanes(s.N), [&](auto lanes) {
+            constexpr int G = decltype(lanes)::value;
+            k_pair_hourglass<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, ucur);
+        });
+    with_lanes(row_lanes(s.N), [&](auto lanes) {
         constexpr int G = decltype(lanes)::value;
         const unsigned grid = nblk(s.N, STEP_THREADS / G);
-        k_pass1_fp64<G><<<grid, STEP_THREADS, 0, st>>>(s, c);
-        if (ev) cudaEventRecord(ev[1], st);
-        if (cfg.hg_alpha != 0.0) k_pass2_fp64<G, true><<<grid, STEP_THREADS, 0, st>>>(s, c);
+        if (hg) k_pass2_fp64<G, true><<<grid, STEP_THREADS, 0, st>>>(s, c);
         else k_pass2_fp64<G, false><<<grid, STEP_THREADS, 0, st>>>(s, c);
-    };
-    with_lanes(s.N, run);
+    });
     if (ev) cudaEventRecord(ev[2], st);
     return cudaGetLastError();
 }
 
-cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, cudaStream_t st)
+cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, int64_t *uoff,
+                             int64_t *scan_tmp, int32_t *id, cudaStream_t st)
 {
-    with_lanes(s.N, [&](auto lanes) {
+    cudaError_t e = cudaMemsetAsync(uoff + s.N, 0, sizeof(int64_t), st);
+    if (e != cudaSuccess) return e;
+    with_lanes(row_lanes(s.N), [&](auto lanes) {
         constexpr int G = decltype(lanes)::value;
-        k_pair_table<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, 1.0 / h, tab, S0);
+        k_pair_table<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, 1.0 / h, tab, S0, uoff);
     });
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = scan_exclusive_i64(uoff, s.N + 1, scan_tmp, st)) != cudaSuccess) return e;
+    k_pair_id<<<nblk(4 * s.N, STEP_THREADS), STEP_THREADS, 0, st>>>(s, uoff, id);
     return cudaGetLastError();
 }
 

@@ -99,6 +99,9 @@ struct DevState {
     // {g = V_j W'/r X_ij, k = (E_i + E_j) V_j W / X_ij^2}, and S0_i = sum_j g_ij (null: formed in place)
     const double4_32a *ptab = nullptr;  // nnz
     const double *ps0 = nullptr;    // N*3
+    const int64_t *puoff = nullptr; // N+1 number of unordered pairs (i, j > i) before row i
+    const int32_t *pid = nullptr;   // nnz number of the entry's unordered pair
+    double4_32a *pw = nullptr;      // nnz / 2 hourglass vectors of the unordered pairs, rewritten each step
 };
 
 // The pass-2 record is tiled by 32 particles: component k (0..5) of particle j
@@ -229,7 +232,8 @@ __host__ __device__ inline void wall_contact(double Xz, double &uz, double &vz)
 // ev: null, or 3 events recorded before pass 1, between the passes and after pass 2
 cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucur, int dcur,
                              int64_t step_index, cudaStream_t st, cudaEvent_t *ev);
-cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, cudaStream_t st);
+cudaError_t build_pair_table(const DevState &s, double h, double4_32a *tab, double *S0, int64_t *uoff,
+                             int64_t *scan_tmp, int32_t *id, cudaStream_t st);
 cudaError_t launch_material_point_value(const DevMat &m, double dt, int64_t n, const double *deps,
                                         const double *J, double *state, cudaStream_t st);
 cudaError_t launch_export_sym(const double *src6, double *dst9, int64_t N, cudaStream_t st);
