@@ -277,7 +277,10 @@ int tlsph_destroy(tlsph_ctx *ctx);
  * 7 as 1 capped for five resident blocks; 8 as 7 with rows 0 and 1 of the
  * stress term formed by packed FP32x2 operations; block size at most 128 for
  * 4 to 8),
- * plan[3] its block size (multiples of 32 up to 256).  Every plan computes
+ * plan[3] its block size (multiples of 32 up to 256).  On contexts of less
+ * than 100,000 particles (pass 1) or 50,000 (pass 2) the pass-1 forms 4 and 5
+ * and the pass-2 form 4 deal each row to 2 to 16 threads, in blocks of 128
+ * whatever the plan's block size.  Every plan computes
  * the same method; sums over a row are grouped differently, so results
  * differ only by FP32 rounding.  n must be 4.  TLSPH_ERR_ARG for a plan out
  * of range.  A new mixed context starts with (4, 64, 4, 128).  The FP64 path

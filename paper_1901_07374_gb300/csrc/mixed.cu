@@ -40,6 +40,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tlsph_device.cuh"
 #include "tlsph_internal.cuh"
@@ -295,17 +296,19 @@ __global__ void k_ell_fill(const int64_t *row_ptr, const int32_t *col, int64_t N
     for (int k = 0; k < wv; ++k) o[32 * k + lane] = k < n ? col[b + k] : pad;
 }
 
-// aligned slice: slots in groups of U; CLAMP replaces an index outside the
-// particle range (only ever a masked slot) by alt
-template <int U, bool CLAMP, class Body>
+// aligned slice: slots in groups of U, every L-th group from group `sub` on
+// (L lanes share a row); CLAMP replaces an index outside the particle range
+// (only ever a masked slot) by alt
+template <int U, bool CLAMP, int L, class Body>
 __device__ __forceinline__ void aligned_slots(const int32_t *__restrict__ base, int W, int lane, int ii, int alt,
-                                              int N, Body &&body)
+                                              int N, int sub, Body &&body)
 {
     const int T = 32 * ((W + 31) / 32);
     const uint32_t *__restrict__ mk = reinterpret_cast<const uint32_t *>(base) + T + lane;
     uint32_t bits = 0;
-    for (int k = 0; k < W; k += U) {
-        if ((k & 31) == 0) bits = mk[k];
+    for (int k = L > 1 ? U * sub : 0; k < W; k += U * L) {
+        if (L > 1) bits = mk[k & ~31] >> (k & 31);
+        else if ((k & 31) == 0) bits = mk[k];
         int o[U];
         // the table is 128-byte aligned and k a multiple of U: one 8- or 16-byte load for the group
         if (U == 2) {
@@ -330,7 +333,7 @@ __device__ __forceinline__ void aligned_slots(const int32_t *__restrict__ base, 
             j[u] = (CLAMP && ju >= (unsigned)N) ? alt : (int)ju;
             w[u] = (bits & (1u << u)) ? 0.0f : SLOT_PAD_Q;
         }
-        bits >>= U;
+        if (L == 1) bits >>= U;
         body(j, w, k);
     }
 }
@@ -340,9 +343,10 @@ __device__ __forceinline__ void aligned_slots(const int32_t *__restrict__ base, 
 // (whose j is a valid particle other than i, so its terms are finite).  The
 // pair terms add qpad to the kernel argument q = r / h: a padding slot lands
 // outside the kernel's support (q >= 2), where W and W' are exactly zero, so
-// its terms vanish without a weight multiply.
-template <int U, class Body>
-__device__ __forceinline__ void for_slots(const DevState &s, int64_t i, Body &&body)
+// its terms vanish without a weight multiply.  With L > 1 the row's groups are
+// dealt to L lanes and this is the turn of lane `sub`.
+template <int U, int L = 1, class Body>
+__device__ __forceinline__ void for_slots(const DevState &s, int64_t i, int sub, Body &&body)
 {
     const int64_t g = i >> 5;
     const int lane = (int)(i & 31);
@@ -351,11 +355,11 @@ __device__ __forceinline__ void for_slots(const DevState &s, int64_t i, Body &&b
     const int alt = i == 0 ? 1 : (int)i - 1;
     if (wv < 0) {
         const int W = (~wv) & 0xffffff;
-        if ((~wv) >> 24) aligned_slots<U, true>(base, W, lane, (int)i, alt, (int)s.N, body);
-        else aligned_slots<U, false>(base, W, lane, (int)i, alt, (int)s.N, body);
+        if ((~wv) >> 24) aligned_slots<U, true, L>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
+        else aligned_slots<U, false, L>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
     } else {
         const int32_t *__restrict__ cp = base + lane;
-        for (int k = 0; k < wv; k += U) {
+        for (int k = L > 1 ? U * sub : 0; k < wv; k += U * L) {
             int j[U];
             float w[U];
 #pragma unroll
@@ -581,6 +585,11 @@ __device__ __forceinline__ void load_u1(const DevState &s, const MixConst &c, in
     u2 = (float)un[3 * i + 2] * c.inv_unit_f;
 }
 
+__device__ __forceinline__ void epi1_slow(const DevState &s, const MixConst &c, int64_t i);
+
+// QUEUE: a particle beyond the FP32 screen is left to k_epi1_slow; otherwise
+// its FP64 update follows at once in the same thread
+template <bool QUEUE = true>
 __device__ __forceinline__ void epi1_mixed(const DevState &s, const MixConst &c, int64_t i, const float *keep)
 {
     const double *__restrict__ Dn = s.D[c.dcur];
@@ -668,8 +677,12 @@ __device__ __forceinline__ void epi1_mixed(const DevState &s, const MixConst &c,
         // the FP64 update finishes this particle (k_epi1_slow): hand it the strain increment
 #pragma unroll
         for (int k = 0; k < 6; ++k) s.fsum[k * N + i] = dh[k];
-        const uint32_t q = atomicAdd(&s.slowq_n[c.step_index & 1], 1u);
-        s.slowq[q] = (int32_t)i;
+        if (QUEUE) {
+            const uint32_t q = atomicAdd(&s.slowq_n[c.step_index & 1], 1u);
+            s.slowq[q] = (int32_t)i;
+        } else {
+            epi1_slow(s, c, i);
+        }
         if (st) atomicOr(s.status, st);
         return;
     }
@@ -798,8 +811,8 @@ __device__ __forceinline__ void pair1(const MixConst &c, const int4 oi, const fl
 // thread per row over the sliced neighbour lists, U pairs in flight; with TAB
 // (four pairs in flight) the weights come from the per-slot table, one float4
 // per group of four slots, laid out [group][lane] within the slice
-template <int U, bool TAB = false>
-__device__ __forceinline__ void gather1_row(const DevState &s, const MixConst &c, int64_t i, float *m)
+template <int U, bool TAB = false, int L = 1>
+__device__ __forceinline__ void gather1_row(const DevState &s, const MixConst &c, int64_t i, float *m, int sub = 0)
 {
     const int4 oi = s.xo[i];
     const float4 vi = s.r1[i];
@@ -808,7 +821,7 @@ __device__ __forceinline__ void gather1_row(const DevState &s, const MixConst &c
     if constexpr (TAB) {
         static_assert(U == 4, "the weight table holds groups of four slots");
         const float4 *__restrict__ tb = s.w1t + s.w1t_off[i >> 5] + (i & 31);
-        for_slots<U>(s, i, [&](const int *j, const float *, int k) {
+        for_slots<U, L>(s, i, sub, [&](const int *j, const float *, int k) {
             int4 o[U];
             float4 v[U];
 #pragma unroll
@@ -820,7 +833,7 @@ __device__ __forceinline__ void gather1_row(const DevState &s, const MixConst &c
         });
         return;
     }
-    for_slots<U>(s, i, [&](const int *j, const float *w, int) {
+    for_slots<U, L>(s, i, sub, [&](const int *j, const float *w, int) {
         int4 o[U];
         float4 v[U];
 #pragma unroll
@@ -1115,13 +1128,13 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
 }
 
 // pass-2 pair sums of row i over its slots, U pairs in flight
-template <bool HG, int U, bool PK = false>
-__device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c, int64_t i, float *acc)
+template <bool HG, int U, bool PK = false, int L = 1>
+__device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c, int64_t i, float *acc, int sub = 0)
 {
     const Row2 w = load_row2<HG>(s, c, i);
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-    for_slots<U>(s, i, [&](const int *j, const float *wm, int) {
+    for_slots<U, L>(s, i, sub, [&](const int *j, const float *wm, int) {
 #pragma unroll
         for (int u = 0; u < U; ++u) pair2<HG, PK>(s, c, w, j[u], wm[u], acc);
     });
@@ -1224,6 +1237,106 @@ __global__ void __launch_bounds__(128, 9) k_gather1_mixed_t4w(DevState s, MixCon
     gather1_row<4, true>(s, c, i, m);
 #pragma unroll
     for (int k = 0; k < 9; ++k) s.fsum[k * s.N + i] = m[k];
+}
+
+// ------------------------------------------------------------------ several lanes per row
+// Small contexts: one thread per row leaves a specimen of a few thousand
+// particles on a few dozen blocks whose threads walk about 118 slots in series
+// (65 us per step at 2048 particles, all of it latency).  Here L lanes share a
+// row's slot groups, a block of 128 threads holds 128 / L rows and leaves their
+// sums in shared memory, and its first 128 / L threads run the per-particle
+// part, the FP64 update of Algorithms 1 and 2 included (FUSED): a step is two
+// launches instead of four.  At 43,000 particles and more the lanes of a warp
+// then gather from L separate runs of particles, which costs more than the
+// shorter rows give.  us per step, one thread per row against L = 2 / 4 / 8 /
+// 16 (fused):
+//   2048     60 | 35 / 27 / 25 / 19        25,000   80 | 49 / 53 / 68 / 82
+//   5148     68 | 41 / 32 / 27 / 27        42,693  106 | 82 / 104 / 125 / 152 (plastic flow)
+//   12,000   70 | 42 / 33 / 39 / 47        64,200   97 | 98 / 121 / 156 / 197
+// Pass 1 alone still gains from two lanes up to 100,000 particles, with its
+// per-particle part in kernels of its own (Taylor cylinder of 60,000: 59 -> 53).
+struct RowLanes {
+    int pass1, pass2;   // lanes per row; 1: the plan's own kernels
+    bool fused;         // pass 1 with the per-particle part in the same kernel
+};
+static RowLanes row_lanes(int64_t N)
+{
+    if (N < 4096) return { 16, 16, true };
+    if (N < 8192) return { 8, 8, true };
+    if (N < 20000) return { 4, 4, true };
+    if (N < 50000) return { 2, 2, true };
+    return { N < 100000 ? 2 : 1, 1, false };
+}
+template <class F>
+static void with_lanes(int lanes, F &&f)
+{
+    if (lanes == 2) f(std::integral_constant<int, 2>());
+    else if (lanes == 4) f(std::integral_constant<int, 4>());
+    else if (lanes == 8) f(std::integral_constant<int, 8>());
+    else f(std::integral_constant<int, 16>());
+}
+
+// sum over the L lanes of a row (every lane of the warp takes part)
+template <int L>
+__device__ __forceinline__ float lane_sum(float x)
+{
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+template <int L, bool FUSED>
+__global__ void __launch_bounds__(128) k_pass1_mixed_rows(DevState s, MixConst c)
+{
+    constexpr int ROWS = 128 / L;
+    __shared__ float sums[9][ROWS];
+    const int sub = threadIdx.x % L, slot = threadIdx.x / L;
+    const int64_t row0 = (int64_t)blockIdx.x * ROWS, i = row0 + slot;
+    float m[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = 0.0f;
+    if (i < s.N) gather1_row<4, false, L>(s, c, i, m, sub);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = lane_sum<L>(m[k]);
+    if (!FUSED) {
+        if (sub == 0 && i < s.N)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) s.fsum[k * s.N + i] = m[k];
+        return;
+    }
+    if (sub == 0)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) sums[k][slot] = m[k];
+    __syncthreads();
+    // this form leaves no queue behind: the other forms find it empty
+    if (blockIdx.x == 0 && threadIdx.x == 0) s.slowq_n[0] = s.slowq_n[1] = 0u;
+    if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = sums[k][threadIdx.x];
+    epi1_mixed<false>(s, c, row0 + threadIdx.x, m);
+}
+
+template <bool HG, int L>
+__global__ void __launch_bounds__(128) k_pass2_mixed_rows(DevState s, MixConst c)
+{
+    constexpr int ROWS = 128 / L;
+    __shared__ float sums[9][ROWS];
+    const int sub = threadIdx.x % L, slot = threadIdx.x / L;
+    const int64_t row0 = (int64_t)blockIdx.x * ROWS, i = row0 + slot;
+    float m[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = 0.0f;
+    if (i < s.N) gather2_row<HG, 2, false, L>(s, c, i, m, sub);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        m[k] = lane_sum<L>(m[k]);
+        if (sub == 0) sums[k][slot] = m[k];
+    }
+    __syncthreads();
+    if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = sums[k][threadIdx.x];
+    epi2_mixed<HG>(s, c, row0 + threadIdx.x, m);
 }
 
 // split form of pass 2: a gather kernel with no FP64 epilogue stores the 9
@@ -1383,7 +1496,7 @@ __global__ void __launch_bounds__(256) k_shape_mixed(DevState s, float inv_h, do
     float sm[9], cp[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) sm[k] = cp[k] = 0.0f;
-    for_slots<2>(s, i, [&](const int *j, const float *w, int) {
+    for_slots<2>(s, i, 0, [&](const int *j, const float *w, int) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const float3 d = xdiff(s.xo[j[u]], oi);
@@ -1463,7 +1576,7 @@ __global__ void __launch_bounds__(256) k_w1t_fill(DevState s, float inv_h)
         return;
     }
     const int4 oi = s.xo[i];
-    for_slots<4>(s, i, [&](const int *j, const float *w, int k) {
+    for_slots<4>(s, i, 0, [&](const int *j, const float *w, int k) {
         float t[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) t[u] = w1_weight(xdiff(s.xo[j[u]], oi), inv_h, w[u]);
@@ -1505,6 +1618,7 @@ int mixed_slow_grid()
 //           5 = as 3 with registers capped for 8 blocks of 128;  6 = as 1 with registers capped for 7 blocks of 128;
 //           7 = as 1 with registers capped for 5 blocks of 128;  8 = as 7 with packed FP32x2 stress rows
 // block sizes are multiples of 32 up to 256 (128 for the fused warp forms and pass-2 forms 4 to 8).
+// Pass-1 forms 4 and 5 and pass-2 form 4 share a row between several lanes on small contexts (row_lanes).
 cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t st, cudaEvent_t *ev)
 {
     const MixConst c = make_mix_const(ctx, step_index);
@@ -1513,6 +1627,16 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
     const bool hg = ctx.cfg.hg_alpha != 0.0;
     const int64_t rows32 = (s.N + 31) / 32 * 32;
     if (ev) cudaEventRecord(ev[0], st);
+    const RowLanes rl = row_lanes(s.N);
+    const bool rows1 = (v1 == 4 || v1 == 5) && rl.pass1 > 1, fused1 = rows1 && rl.fused;
+    if (rows1) {
+        with_lanes(rl.pass1, [&](auto lanes) {
+            constexpr int L = decltype(lanes)::value;
+            if (fused1) k_pass1_mixed_rows<L, true><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+            else k_pass1_mixed_rows<L, false><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+        });
+        if (!fused1) k_epi1_mixed<<<nb(s.N, 128), 128, 0, st>>>(s, c);
+    } else
     switch (v1) {
     case 1: k_pass1_mixed_t<<<nb(s.N, b1), b1, 0, st>>>(s, c); break;
     case 2:
@@ -1533,9 +1657,15 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
         break;
     default: k_pass1_mixed<<<nb(rows32, MIX_THREADS), MIX_THREADS, 0, st>>>(s, c); break;
     }
-    k_epi1_slow<<<ctx.slow_grid, 128, 0, st>>>(s, c);
+    if (!fused1) k_epi1_slow<<<ctx.slow_grid, 128, 0, st>>>(s, c);
     if (ev) cudaEventRecord(ev[1], st);
-    if (v2 == 1) {
+    if (v2 == 4 && rl.pass2 > 1) {
+        with_lanes(rl.pass2, [&](auto lanes) {
+            constexpr int L = decltype(lanes)::value;
+            if (hg) k_pass2_mixed_rows<true, L><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+            else k_pass2_mixed_rows<false, L><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+        });
+    } else if (v2 == 1) {
         if (hg) k_pass2_mixed_t<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_t<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
     } else if (v2 == 3) {
@@ -1571,8 +1701,6 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
     if (ev) cudaEventRecord(ev[2], st);
     return cudaGetLastError();
 }
-
-int mixed_kernels_per_step(const tlsph_ctx &ctx) { return (ctx.plan[0] >= 2 ? 2 : 1) + 1 + (ctx.plan[2] == 2 ? 2 : 1); }
 
 cudaError_t mixed_sync_to_fp64(tlsph_ctx &ctx, int field, cudaStream_t st)
 {

@@ -323,7 +323,6 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
 int mixed_slow_grid();
 // compensated mixed state -> FP64 arrays for one field or all (-1)
 cudaError_t mixed_sync_to_fp64(tlsph_ctx &ctx, int field, cudaStream_t st);
-int mixed_kernels_per_step(const tlsph_ctx &ctx);
 void mixed_release(tlsph_ctx &ctx);
 
 }  // namespace tlsph
