@@ -29,7 +29,7 @@ struct Layout {
     size_t ep, epdot, dinit, por, e, D0, D1, force, fail, status, mats, col, diag, inscan;
     size_t xo, s0, linv32, r1, r2, fsum, ell_off, ell_w;
     size_t Fh, Fl, sdh, sdl, sigf, slowq, slowq_n;
-    size_t scratch, cell_start, cell_cursor, cell_items, scan_tmp, xf;
+    size_t scratch, cell_start, slot, sorted, scan_tmp;
     size_t perm, iperm, stX, stvol, stmat, stbcm, stbcv, stf0;   // order, its inverse + staged caller-order inputs
     size_t overlay_end, ell;
     size_t total;
@@ -177,11 +177,10 @@ Layout make_layout(int64_t N, int64_t nnz_cap, bool mixed)
     L.stbcm = s.take(n);
     L.stbcv = s.take(3 * n * d);
     L.stf0 = s.take(n * d);
-    L.cell_start = s.take((size_t)(L.max_cells + 1) * sizeof(int64_t));
-    L.cell_cursor = s.take((size_t)L.max_cells * sizeof(int64_t));
-    L.cell_items = s.take(n * sizeof(int32_t));
+    L.cell_start = s.take((size_t)(L.max_cells + 1) * sizeof(int32_t));
+    L.slot = s.take(n * sizeof(int32_t));
+    L.sorted = s.take(n * sizeof(float4));
     L.scan_tmp = s.take(L.scan_elems * sizeof(int64_t));
-    L.xf = s.take(n * 16);
     c.off = std::max(state_end, s.off);
     L.overlay_end = c.off;
     L.col = c.take((size_t)std::max<int64_t>(nnz_cap, 1) * sizeof(int32_t));
@@ -611,8 +610,8 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
     const CellGrid grid = cell_grid_from_bounds(lo3, hi3, N, cfg->rc);         // internal order
     const CellGrid sgrid = cell_grid_from_bounds(lo3, hi3, N, cfg->rc, 2);     // neighbour search
     if (grid.ncells > L.max_cells || sgrid.ncells > L.max_cells) return bail(TLSPH_ERR_ARG, "cell grid exceeds its bound");
-    Scratch sc{ at<int64_t>(base, L.cell_start), at<int64_t>(base, L.cell_cursor), at<int32_t>(base, L.cell_items),
-                at<int64_t>(base, L.scan_tmp), L.scan_elems, at<float4>(base, L.xf) };
+    Scratch sc{ at<int32_t>(base, L.cell_start), at<int32_t>(base, L.slot), at<float4>(base, L.sorted),
+                at<int64_t>(base, L.scan_tmp), L.scan_elems };
     // ---- internal order (brick-major cells, caller index inside a cell) and the gather into it
     const bool line_order = (cfg->flags & TLSPH_FLAG_LINE_ORDER) != 0;
     ctx->reordered = (cfg->flags & (TLSPH_FLAG_SPATIAL_ORDER | TLSPH_FLAG_LINE_ORDER)) != 0;

