@@ -350,7 +350,7 @@ __device__ __forceinline__ void epi1_fp64(const DevState &s, const StepConst &c,
     mp.e = s.e[i];
     mp.failed = 0;
     const DevMat &mat = s.mats[s.mat[i]];
-    st |= material_update<false, true>(mat, c.dt, de, J, mp);
+    st |= material_update<true>(mat, c.dt, de, J, mp);
     // internal energy (Eq. conservation3, de/dt = J sigma : d / rho0), trapezoidal in the step with the
     // stress at its start and at its end (zero after a failure), current frame, d scaled by dt below
     double sgn[6];

