@@ -1059,21 +1059,17 @@ int tlsph_set_state(tlsph_ctx *ctx, int field, const void *src, size_t bytes, in
         ctx->steps = v;
         return TLSPH_OK;
     }
-    if (ctx->cfg.precision == TLSPH_PRECISION_MIXED) {
-        e = mixed_sync_to_fp64(*ctx, -1, st);   // bring every FP64 field up to date first
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "mixed export");
-    }
     const int64_t N = ctx->N;
     const int comps = (int)(f.count / (size_t)N);
     const int scomps = f.sym ? 6 : comps;
+    std::vector<unsigned char> tmp;
     if (src_on_device) {
         if (f.sym || ctx->reordered)
             e = launch_permute(src, f.ptr, ctx->perm_dev, N, scomps, (int)f.elem, false, f.sym, st);
         else
             e = cudaMemcpyAsync(f.ptr, src, bytes, cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     } else {
-        std::vector<unsigned char> tmp((size_t)N * scomps * f.elem);
+        tmp.resize((size_t)N * scomps * f.elem);
         const unsigned char *a = static_cast<const unsigned char *>(src);
         for (int64_t k = 0; k < N; ++k) {
             const int64_t i = ctx->reordered ? ctx->perm[k] : k;
@@ -1087,12 +1083,11 @@ int tlsph_set_state(tlsph_ctx *ctx, int field, const void *src, size_t bytes, in
             }
         }
         e = cudaMemcpyAsync(f.ptr, tmp.data(), tmp.size(), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    if (e == cudaSuccess && ctx->cfg.precision == TLSPH_PRECISION_MIXED) {
-        e = mixed_import(*ctx, field, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
+    // a compensated field's FP32 state follows from its FP64 array; the others' FP64 arrays are only refreshed
+    // when they are read, so nothing is exported here
+    if (e == cudaSuccess && ctx->cfg.precision == TLSPH_PRECISION_MIXED) e = mixed_import(*ctx, field, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);     // src and tmp may go
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set_state");
     ctx->need_predict = true;
     return TLSPH_OK;
