@@ -58,8 +58,10 @@ int64_t ell_capacity(int64_t N, int64_t nnz_cap)
 // Lattice-line order (TLSPH_FLAG_LINE_ORDER): perm[k] = caller index of
 // internal particle k, sorted by the rounded lattice coordinates of the two
 // shorter bounding-box axes, then by the coordinate along the longest axis
-// (quantised to 32 bits over its extent; ties keep the caller order).  A
-// least-significant-digit radix sort (four 16-bit digits) of 64-bit keys.
+// (quantised to 32 bits over its extent; ties keep the caller order).  The
+// host's form of build_line_order, for bodies whose cross-section has more
+// lattice lines than the device scratch: a least-significant-digit radix sort
+// (four 16-bit digits) of 64-bit keys.
 std::vector<int32_t> line_order_perm(const double *X, const double *vol, int64_t N)
 {
     std::vector<int32_t> perm((size_t)N);
@@ -107,6 +109,15 @@ std::vector<int32_t> line_order_perm(const double *X, const double *vol, int64_t
         perm.swap(idx2);
     }
     return perm;
+}
+
+// lattice spacing of the line order: the cube root of the median volume
+double line_spacing(const double *vol, int64_t N, double vmin, double vmax)
+{
+    if (vmin == vmax) return std::cbrt(std::max(vmin, 0.0));
+    std::vector<double> v(vol, vol + N);
+    std::nth_element(v.begin(), v.begin() + N / 2, v.end());
+    return std::cbrt(std::max(v[(size_t)(N / 2)], 0.0));
 }
 
 Layout make_layout(int64_t N, int64_t nnz_cap, bool mixed)
@@ -491,37 +502,6 @@ size_t tlsph_workspace_bytes(const tlsph_config *cfg, int64_t N, int64_t nnz_cap
     return make_layout(N, nnz_cap, cfg->precision == TLSPH_PRECISION_MIXED).total + ALIGN;
 }
 
-// TLSPH_FLAG_AUTO_ORDER: the context in the caller's order, unless fewer than
-// nine in ten of its neighbour slices are aligned (mixed precision only; the
-// FP64 path reads the CSR); then the context is built again in lattice-line
-// order and kept if that aligns more slices, else built once more in the
-// caller's order.
-static int create_auto_order(const tlsph_config *cfg, int64_t N, const double *X, const double *vol,
-                             const int32_t *mat_id, const uint8_t *bc_mask, const double *bc_vel,
-                             const double *f0, void *arena, size_t arena_bytes, int64_t nnz_cap,
-                             void *stream, tlsph_ctx **out)
-{
-    tlsph_config caller = *cfg;
-    caller.flags &= ~TLSPH_FLAG_AUTO_ORDER;
-    int r = tlsph_create(&caller, N, X, vol, mat_id, bc_mask, bc_vel, f0, arena, arena_bytes, nnz_cap, stream, out);
-    if (r != TLSPH_OK || caller.precision != TLSPH_PRECISION_MIXED) return r;
-    int64_t slices = 0, aligned = 0;
-    if (tlsph_neighbor_layout(*out, &slices, &aligned, nullptr, nullptr) != TLSPH_OK || 10 * aligned >= 9 * slices)
-        return TLSPH_OK;
-    tlsph_destroy(*out);
-    *out = nullptr;
-    tlsph_config line = caller;
-    line.flags |= TLSPH_FLAG_LINE_ORDER;
-    r = tlsph_create(&line, N, X, vol, mat_id, bc_mask, bc_vel, f0, arena, arena_bytes, nnz_cap, stream, out);
-    if (r == TLSPH_OK) {
-        int64_t s2 = 0, a2 = 0;
-        if (tlsph_neighbor_layout(*out, &s2, &a2, nullptr, nullptr) == TLSPH_OK && a2 > aligned) return TLSPH_OK;
-        tlsph_destroy(*out);
-        *out = nullptr;
-    }
-    return tlsph_create(&caller, N, X, vol, mat_id, bc_mask, bc_vel, f0, arena, arena_bytes, nnz_cap, stream, out);
-}
-
 int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const double *vol,
                  const int32_t *mat_id, const uint8_t *bc_mask, const double *bc_vel,
                  const double *f0, void *arena, size_t arena_bytes, int64_t nnz_cap,
@@ -532,8 +512,6 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
     if (!out) { g_create_error = "out is NULL"; return TLSPH_ERR_ARG; }
     *out = nullptr;
     if (!valid_config(cfg, why)) { g_create_error = why; return TLSPH_ERR_ARG; }
-    if (cfg->flags & TLSPH_FLAG_AUTO_ORDER)
-        return create_auto_order(cfg, N, X, vol, mat_id, bc_mask, bc_vel, f0, arena, arena_bytes, nnz_cap, stream, out);
     if (N <= 0 || N > INT32_MAX) { g_create_error = "N must be in [1, 2^31)"; return TLSPH_ERR_ARG; }
     if (!X || !vol) { g_create_error = "X and vol are required"; return TLSPH_ERR_ARG; }
     if (arena && ((uintptr_t)arena % ALIGN) != 0) { g_create_error = "arena must be 256-byte aligned"; return TLSPH_ERR_ARG; }
@@ -542,6 +520,7 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
     tlsph_ctx *ctx = new (std::nothrow) tlsph_ctx();
     if (!ctx) { g_create_error = "host allocation failed"; return TLSPH_ERR_NOMEM; }
     ctx->cfg = *cfg;
+    ctx->cfg.flags &= ~TLSPH_FLAG_AUTO_ORDER;      // the order chosen below takes its place
     ctx->N = N;
     ctx->stream = static_cast<cudaStream_t>(stream);
     cudaStream_t st = ctx->stream;
@@ -615,53 +594,84 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
     if (grid.ncells > L.max_cells || sgrid.ncells > L.max_cells) return bail(TLSPH_ERR_ARG, "cell grid exceeds its bound");
     Scratch sc{ at<int32_t>(base, L.cell_start), at<int32_t>(base, L.slot), at<float4>(base, L.sorted),
                 at<int64_t>(base, L.scan_tmp), L.scan_elems };
-    // ---- internal order (brick-major cells, caller index inside a cell) and the gather into it
-    const bool line_order = (cfg->flags & TLSPH_FLAG_LINE_ORDER) != 0;
-    ctx->reordered = (cfg->flags & (TLSPH_FLAG_SPATIAL_ORDER | TLSPH_FLAG_LINE_ORDER)) != 0;
-    ctx->perm_dev = at<int32_t>(base, L.perm);
-    if (line_order) {
-        const std::vector<int32_t> lp = line_order_perm(X, vol, N);
-        CK(cudaMemcpyAsync(ctx->perm_dev, lp.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        CK(cudaStreamSynchronize(st));
-    } else {
-        CK(build_order(stX, N, grid, sc, !ctx->reordered, ctx->perm_dev, st));
-    }
-    CK(launch_gather_inputs(ctx->perm_dev, N, stX, stvol, stmat, stbcm, stbcv, stf0, s, st));
-    // host copies of the order and its inverse (kept empty in caller order: the identity)
-    if (ctx->reordered) {
-        ctx->perm.resize(n);
-        ctx->inv.resize(n);
-        CK(cudaMemcpyAsync(ctx->perm.data(), ctx->perm_dev, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        for (size_t k = 0; k < n; ++k) ctx->inv[ctx->perm[k]] = (int32_t)k;
-    }
-
     const double rc2 = cfg->rc * cfg->rc;
     int64_t *row_ptr = const_cast<int64_t *>(s.row_ptr);
-    CK(build_neighbors_count(s, sgrid, sc, rc2, row_ptr, st));
-    int64_t nnz = 0;
-    CK(cudaMemcpyAsync(&nnz, row_ptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (nnz > INT32_MAX) return bail(TLSPH_ERR_ARG, "more than 2^31 - 1 neighbour pairs");
-    if (arena) {
-        if (nnz > nnz_cap)
-            return bail(TLSPH_ERR_NOMEM, "neighbour capacity too small: need nnz_cap >= " + std::to_string(nnz));
-        s.col = at<int32_t>(base, L.col);
-    } else {
-        // the columns in an allocation of their own, now that their count is known
-        e = cudaMalloc(&ctx->col_mem, (size_t)std::max<int64_t>(nnz, 1) * sizeof(int32_t));
-        if (e != cudaSuccess) { cudaGetLastError(); return bail(TLSPH_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)); }
-        s.col = static_cast<int32_t *>(ctx->col_mem);
-        ctx->nnz_cap = nnz;
+    int64_t *ell_off = const_cast<int64_t *>(s.ell_off);
+    const int64_t ng = (N + 31) / 32;
+    int64_t ell_n = 0;
+    ctx->perm_dev = at<int32_t>(base, L.perm);
+    // the inputs in an internal order (0 or one of the order flags), the neighbour CSR over it and, for a mixed
+    // context, the widths and offsets of its sliced lists; called again when another order is tried
+    auto build_lists = [&](int order) -> int {
+        ctx->reordered = order != 0;
+        if (order == TLSPH_FLAG_LINE_ORDER) {
+            bool done = false;
+            CK(build_line_order(stX, N, lo3, hi3, line_spacing(vol, N, scan.vmin, scan.vmax), sc, L.max_cells,
+                                ctx->perm_dev, &done, st));
+            if (!done) {        // more lattice lines than the scratch has room for
+                const std::vector<int32_t> lp = line_order_perm(X, vol, N);
+                CK(cudaMemcpyAsync(ctx->perm_dev, lp.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+                CK(cudaStreamSynchronize(st));
+            }
+        } else {
+            CK(build_order(stX, N, grid, sc, !ctx->reordered, ctx->perm_dev, st));
+        }
+        CK(launch_gather_inputs(ctx->perm_dev, N, stX, stvol, stmat, stbcm, stbcv, stf0, s, st));
+        // inverse order on the device (caller index -> internal index) for the caller-order reads
+        ctx->inv_dev = nullptr;
+        if (ctx->reordered) {
+            ctx->inv_dev = at<int32_t>(base, L.iperm);
+            CK(launch_invert(ctx->perm_dev, ctx->inv_dev, N, st));
+        }
+        CK(build_neighbors_count(s, sgrid, sc, rc2, row_ptr, st));
+        int64_t nnz = 0;
+        CK(cudaMemcpyAsync(&nnz, row_ptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (nnz > INT32_MAX) return bail(TLSPH_ERR_ARG, "more than 2^31 - 1 neighbour pairs");
+        if (arena) {
+            if (nnz > nnz_cap)
+                return bail(TLSPH_ERR_NOMEM, "neighbour capacity too small: need nnz_cap >= " + std::to_string(nnz));
+            s.col = at<int32_t>(base, L.col);
+        } else if (!ctx->col_mem) {
+            // the columns in an allocation of their own, now that their count (the same in every order) is known
+            e = cudaMalloc(&ctx->col_mem, (size_t)std::max<int64_t>(nnz, 1) * sizeof(int32_t));
+            if (e != cudaSuccess) { cudaGetLastError(); return bail(TLSPH_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)); }
+            s.col = static_cast<int32_t *>(ctx->col_mem);
+            ctx->nnz_cap = nnz;
+        }
+        ctx->nnz = nnz;
+        CK(build_neighbors_fill(s, sgrid, sc, rc2, row_ptr, const_cast<int32_t *>(s.col), st));
+        if (mixed) {
+            CK(cudaMemsetAsync(ell_off + ng, 0, sizeof(int64_t), st));
+            CK(mixed_ell_widths(s, ell_off, st));
+            CK(scan_exclusive_i64(ell_off, ng + 1, sc.scan_tmp, st));
+            CK(cudaMemcpyAsync(&ell_n, ell_off + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+        }
+        return TLSPH_OK;
+    };
+    const int order = cfg->flags & (TLSPH_FLAG_SPATIAL_ORDER | TLSPH_FLAG_LINE_ORDER);
+    if (const int r = build_lists(order)) return r;
+    if (mixed && (cfg->flags & TLSPH_FLAG_AUTO_ORDER)) {
+        // the caller's order, unless fewer than nine in ten of its slices are aligned and lattice lines align more
+        const auto fits = [&] { return !arena || ell_n <= ell_capacity(N, nnz_cap); };
+        std::vector<int32_t> w((size_t)ng);
+        const auto aligned = [&](int64_t &count) {
+            count = 0;
+            cudaError_t err = cudaMemcpyAsync(w.data(), s.ell_w, (size_t)ng * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+            if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+            for (int32_t x : w) count += x < 0;
+            return err;
+        };
+        int64_t a0 = 0, a1 = 0;
+        CK(aligned(a0));
+        if (fits() && 10 * a0 < 9 * ng) {
+            if (const int r = build_lists(TLSPH_FLAG_LINE_ORDER)) return r;
+            CK(aligned(a1));
+            if (fits() && a1 > a0) ctx->cfg.flags |= TLSPH_FLAG_LINE_ORDER;
+            else if (const int r = build_lists(0)) return r;
+        }
     }
-    ctx->nnz = nnz;
-    // inverse order on the device (caller index -> internal index) for the caller-order reads
-    ctx->inv_dev = nullptr;
-    if (ctx->reordered) {
-        ctx->inv_dev = at<int32_t>(base, L.iperm);
-        CK(cudaMemcpyAsync(ctx->inv_dev, ctx->inv.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    }
-    CK(build_neighbors_fill(s, sgrid, sc, rc2, row_ptr, const_cast<int32_t *>(s.col), st));
 
     // ---- mixed: fixed-point positions and the sliced neighbour lists, read by
     // the correction-matrix kernel of a mixed context as by its steps
@@ -684,14 +694,6 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
         CK(mixed_init_positions(s, pk, st));
         ctx->slow_grid = mixed_slow_grid();
         // sliced neighbour lists for the thread-per-row plans
-        const int64_t ng = (N + 31) / 32;
-        int64_t *ell_off = const_cast<int64_t *>(s.ell_off);
-        CK(cudaMemsetAsync(ell_off + ng, 0, sizeof(int64_t), st));
-        CK(mixed_ell_widths(s, ell_off, st));
-        CK(scan_exclusive_i64(ell_off, ng + 1, sc.scan_tmp, st));
-        int64_t ell_n = 0;
-        CK(cudaMemcpyAsync(&ell_n, ell_off + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
         ctx->ell_words = ell_n;
         int32_t *colE = nullptr;
         if (arena) {
@@ -924,6 +926,22 @@ int tlsph_info(const tlsph_ctx *ctx, int64_t *N, int64_t *nnz, int64_t *steps)
     return TLSPH_OK;
 }
 
+// host copies of the internal order and its inverse, made when a host-side
+// transfer first needs them
+static cudaError_t host_order(tlsph_ctx *ctx)
+{
+    if (!ctx->reordered || !ctx->perm.empty()) return cudaSuccess;
+    const size_t n = (size_t)ctx->N;
+    std::vector<int32_t> perm(n);
+    cudaError_t e = cudaMemcpyAsync(perm.data(), ctx->perm_dev, n * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return e;
+    ctx->inv.resize(n);
+    for (size_t k = 0; k < n; ++k) ctx->inv[perm[k]] = (int32_t)k;
+    ctx->perm.swap(perm);
+    return cudaSuccess;
+}
+
 // neighbour CSR in caller indices (rows of caller particles, columns mapped
 // back and sorted ascending) from the internal CSR
 static cudaError_t caller_csr(tlsph_ctx *ctx, std::vector<int64_t> &rp, std::vector<int32_t> &col)
@@ -931,7 +949,8 @@ static cudaError_t caller_csr(tlsph_ctx *ctx, std::vector<int64_t> &rp, std::vec
     const int64_t N = ctx->N, nnz = ctx->nnz;
     std::vector<int64_t> rpi(N + 1);
     std::vector<int32_t> ci(nnz);
-    cudaError_t e = cudaMemcpyAsync(rpi.data(), ctx->s.row_ptr, (N + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost,
+    cudaError_t e = host_order(ctx);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(rpi.data(), ctx->s.row_ptr, (N + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost,
                                     ctx->stream);
     if (e == cudaSuccess && nnz > 0)
         e = cudaMemcpyAsync(ci.data(), ctx->s.col, nnz * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream);
@@ -1015,7 +1034,8 @@ int tlsph_get_state(tlsph_ctx *ctx, int field, void *dst, size_t bytes, int dst_
         // caller's order on the host (faster here than the driver's own
         // staging into pages the caller has not touched yet)
         std::vector<unsigned char> tmp(sbytes);
-        e = cudaMemcpyAsync(tmp.data(), f.ptr, sbytes, cudaMemcpyDeviceToHost, st);
+        e = host_order(ctx);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(tmp.data(), f.ptr, sbytes, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e == cudaSuccess && plain) {
             memcpy(dst, tmp.data(), sbytes);
@@ -1069,6 +1089,8 @@ int tlsph_set_state(tlsph_ctx *ctx, int field, const void *src, size_t bytes, in
         else
             e = cudaMemcpyAsync(f.ptr, src, bytes, cudaMemcpyDeviceToDevice, st);
     } else {
+        e = host_order(ctx);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "set_state order");
         tmp.resize((size_t)N * scomps * f.elem);
         const unsigned char *a = static_cast<const unsigned char *>(src);
         for (int64_t k = 0; k < N; ++k) {

@@ -453,6 +453,120 @@ __global__ void k_identity(int32_t *perm, int64_t N)
     if (i < N) perm[i] = (int32_t)i;
 }
 
+// Lattice-line order (TLSPH_FLAG_LINE_ORDER): perm[k] = caller index of
+// internal particle k, by the rounded lattice coordinates of the two shorter
+// axes, then by the coordinate along the longest axis (quantised to 32 bits
+// over its extent), ties by caller index.  Particles are counted and scattered
+// into their lines, then a block sorts each line by (quantised coordinate,
+// caller index), a key of its own per particle, so the order is unique.  The
+// host's radix sort took 1.5 ms at 60,000 particles and 38 ms at 1.02 million.
+struct LineArgs {
+    double lo[3], inv, qL;
+    int a, b, L;
+    int64_t nb;
+};
+
+__device__ __forceinline__ int64_t line_of(const LineArgs &g, const double *x)
+{
+    return llround((x[g.a] - g.lo[g.a]) * g.inv) * g.nb + llround((x[g.b] - g.lo[g.b]) * g.inv);
+}
+
+__global__ void k_line_count(const double *X, int64_t N, LineArgs g, int32_t *count, int32_t *slot)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    slot[i] = atomicAdd(&count[line_of(g, X + 3 * i)], 1);
+}
+
+__global__ void k_line_scatter(const double *X, int64_t N, LineArgs g, const int32_t *start, const int32_t *slot,
+                               uint64_t *key)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const double t = fmin(4294967295.0, fmax(0.0, floor((X[3 * i + g.L] - g.lo[g.L]) * g.qL)));
+    key[start[line_of(g, X + 3 * i)] + slot[i]] = ((uint64_t)t << 32) | (uint64_t)i;
+}
+
+// ascending sort of n keys by one block: the bitonic network whose every
+// comparison puts the smaller key first (the first step of a merge mirrors its
+// block), which takes any n: partners past the end are skipped
+__device__ __forceinline__ void block_sort(uint64_t *v, int n)
+{
+    for (int size = 2; (size >> 1) < n; size <<= 1)
+        for (int d = size >> 1; d > 0; d >>= 1) {
+            __syncthreads();
+            for (int k = threadIdx.x; 2 * k < n + 2 * d; k += blockDim.x) {
+                const int i = 2 * k - (k & (d - 1));                       // lower index of the k-th comparison
+                const int j = d == size >> 1 ? (i ^ (size - 1)) : i + d;
+                if (j < n && v[j] < v[i]) {
+                    const uint64_t t = v[i];
+                    v[i] = v[j];
+                    v[j] = t;
+                }
+            }
+        }
+    __syncthreads();
+}
+
+constexpr int LINE_SMEM = 2048;
+__global__ void __launch_bounds__(256) k_line_sort(const int32_t *start, uint64_t *key, int32_t *perm, int64_t nlines)
+{
+    __shared__ uint64_t sh[LINE_SMEM];
+    for (int64_t line = blockIdx.x; line < nlines; line += gridDim.x) {
+        const int b = start[line], n = start[line + 1] - b;
+        uint64_t *v = key + b;
+        if (n <= LINE_SMEM) {
+            __syncthreads();
+            for (int k = threadIdx.x; k < n; k += blockDim.x) sh[k] = v[k];
+            v = sh;
+        }
+        block_sort(v, n);
+        for (int k = threadIdx.x; k < n; k += blockDim.x) perm[b + k] = (int32_t)(v[k] & 0xffffffffu);
+    }
+}
+
+cudaError_t build_line_order(const double *X, int64_t N, const double *lo, const double *hi, double d, const Scratch &sc,
+                             int64_t max_lines, int32_t *perm, bool *done, cudaStream_t st)
+{
+    LineArgs g{};
+    for (int k = 0; k < 3; ++k) g.lo[k] = lo[k];
+    for (int k = 1; k < 3; ++k)
+        if (hi[k] - lo[k] > hi[g.L] - lo[g.L]) g.L = k;
+    g.a = (g.L + 1) % 3;
+    g.b = (g.L + 2) % 3;
+    g.inv = d > 0.0 ? 1.0 / d : 0.0;
+    const double ext = hi[g.L] - lo[g.L];
+    g.qL = ext > 0.0 ? 4294967295.0 / ext : 0.0;
+    const double na = (hi[g.a] - lo[g.a]) * g.inv + 1.0, nb = (hi[g.b] - lo[g.b]) * g.inv + 1.0;
+    *done = (na + 1.0) * (nb + 1.0) < (double)max_lines;
+    if (!*done) return cudaSuccess;
+    g.nb = llround((hi[g.b] - lo[g.b]) * g.inv) + 1;
+    const int64_t lines = (llround((hi[g.a] - lo[g.a]) * g.inv) + 1) * g.nb;
+    uint64_t *key = reinterpret_cast<uint64_t *>(sc.sorted);
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(sc.cell_start, 0, (lines + 1) * sizeof(int32_t), st)) != cudaSuccess) return e;
+    k_line_count<<<blocks_for(N, 256), 256, 0, st>>>(X, N, g, sc.cell_start, sc.slot);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = scan_exclusive(sc.cell_start, lines + 1, reinterpret_cast<int32_t *>(sc.scan_tmp), st)) != cudaSuccess)
+        return e;
+    k_line_scatter<<<blocks_for(N, 256), 256, 0, st>>>(X, N, g, sc.cell_start, sc.slot, key);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_line_sort<<<(unsigned)std::min<int64_t>(lines, 152 * 8), 256, 0, st>>>(sc.cell_start, key, perm, lines);
+    return cudaGetLastError();
+}
+
+__global__ void k_invert(const int32_t *perm, int32_t *inv, int64_t N)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < N) inv[perm[k]] = (int32_t)k;
+}
+
+cudaError_t launch_invert(const int32_t *perm, int32_t *inv, int64_t N, cudaStream_t st)
+{
+    k_invert<<<blocks_for(N, 256), 256, 0, st>>>(perm, inv, N);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- input scan
 // Every block takes a contiguous range of particles, every thread a strided
 // part of it; the block reduction and the final one run in a fixed order, so
@@ -460,6 +574,8 @@ __global__ void k_identity(int32_t *perm, int64_t N)
 __device__ __forceinline__ void inscan_init(InputScanDev &a)
 {
     for (int k = 0; k < 3; ++k) { a.lo[k] = INFINITY; a.hi[k] = -INFINITY; a.vsum[k] = 0.0; }
+    a.vmin = INFINITY;
+    a.vmax = -INFINITY;
     a.mats = 0ull;
     a.bad = 0u;
     a.pad = 0u;
@@ -471,6 +587,8 @@ __device__ __forceinline__ void inscan_merge(InputScanDev &a, const InputScanDev
         a.hi[k] = fmax(a.hi[k], b.hi[k]);
         a.vsum[k] += b.vsum[k];
     }
+    a.vmin = fmin(a.vmin, b.vmin);
+    a.vmax = fmax(a.vmax, b.vmax);
     a.mats |= b.mats;
     a.bad |= b.bad;
 }
@@ -483,6 +601,8 @@ __device__ __forceinline__ void inscan_warp(InputScanDev &a)
             b.hi[k] = __shfl_xor_sync(0xffffffffu, a.hi[k], o);
             b.vsum[k] = __shfl_xor_sync(0xffffffffu, a.vsum[k], o);
         }
+        b.vmin = __shfl_xor_sync(0xffffffffu, a.vmin, o);
+        b.vmax = __shfl_xor_sync(0xffffffffu, a.vmax, o);
         b.mats = __shfl_xor_sync(0xffffffffu, a.mats, o);
         b.bad = __shfl_xor_sync(0xffffffffu, a.bad, o);
         inscan_merge(a, b);
@@ -512,6 +632,8 @@ __global__ void __launch_bounds__(256) k_scan_inputs(const double *X, const doub
     for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
         const double vv = vol[i];
         if (!(vv > 0.0 && isfinite(vv))) a.bad |= INSCAN_BAD_VOL;
+        a.vmin = fmin(a.vmin, vv);
+        a.vmax = fmax(a.vmax, vv);
         for (int k = 0; k < 3; ++k) {
             const double c = X[3 * i + k];
             if (!isfinite(c)) a.bad |= INSCAN_BAD_X;

@@ -190,12 +190,19 @@ cudaError_t build_neighbors_fill(const DevState &s, const CellGrid &g, const Scr
 // keep = identity
 cudaError_t build_order(const double *X_user, int64_t N, const CellGrid &g, const Scratch &sc, bool keep,
                         int32_t *perm, cudaStream_t st);
+// lattice-line order on the device; *done = false (nothing written) when the cross-section has too many lattice
+// lines of spacing d for the scratch (max_lines)
+cudaError_t build_line_order(const double *X, int64_t N, const double *lo, const double *hi, double d, const Scratch &sc,
+                             int64_t max_lines, int32_t *perm, bool *done, cudaStream_t st);
+// inv[perm[k]] = k
+cudaError_t launch_invert(const int32_t *perm, int32_t *inv, int64_t N, cudaStream_t st);
 // create-time scan of the staged caller-order inputs: bounding box, the
 // materials in use, the sum of the initial velocities and validity flags;
 // a deterministic reduction over INSCAN_BLOCKS blocks whose result lands in
 // parts[0]
 struct InputScanDev {
     double lo[3], hi[3], vsum[3];
+    double vmin, vmax;         // smallest and largest volume
     unsigned long long mats;   // bit m: material m in use
     unsigned int bad;          // INSCAN_BAD_* bits
     unsigned int pad;
