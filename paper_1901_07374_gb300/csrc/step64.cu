@@ -611,13 +611,8 @@ __global__ void k_apply_grip(DevState s, double t)
     apply_bc(s, i, s.fail[i], t, s.v + 3 * i);
 }
 
-__global__ void k_material_point(const DevMat m, double dt, int64_t n, const double *deps, const double *J,
-                                 double *state)
+__device__ __forceinline__ void point_update(const DevMat &m, double dt, const double *e, double J, double *x)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const double *e = deps + 9 * t;
-    double *x = state + 16 * t;
     const double de[6] = { e[0], e[4], e[8], 0.5 * (e[1] + e[3]), 0.5 * (e[5] + e[7]), 0.5 * (e[2] + e[6]) };
     MPState mp;
     mp.sd[0] = x[0]; mp.sd[1] = x[4]; mp.sd[2] = x[8];
@@ -625,10 +620,51 @@ __global__ void k_material_point(const DevMat m, double dt, int64_t n, const dou
     mp.sm = x[9]; mp.ep = x[10]; mp.epdot = x[11]; mp.dinit = x[12]; mp.D = x[13]; mp.f = x[14];
     mp.e = 0.0;        // the material-point driver holds the internal energy at zero
     mp.failed = x[15] != 0.0;
-    material_update(m, dt, de, J[t], mp);
+    material_update<true>(m, dt, de, J, mp);
     sym_to_full(mp.sd, x);
     x[9] = mp.sm; x[10] = mp.ep; x[11] = mp.epdot; x[12] = mp.dinit; x[13] = mp.D; x[14] = mp.f;
     x[15] = mp.failed ? 1.0 : 0.0;
+}
+
+// whether the point yields, by FP32 (only the order of the work depends on it)
+__device__ __forceinline__ bool point_yields_f(const DevMat &m, const double *e, double J, const double *x)
+{
+    if (x[15] != 0.0) return false;
+    const float D = (float)x[13], g2 = 2.0f * m.Gf * (1.0f - D);
+    const float d0 = (float)e[0], d1 = (float)e[4], d2 = (float)e[8], tr = (d0 + d1 + d2) * (1.0f / 3.0f);
+    const float a = (float)x[0] + g2 * (d0 - tr), b = (float)x[4] + g2 * (d1 - tr), c = (float)x[8] + g2 * (d2 - tr);
+    const float p = 0.5f * ((float)x[1] + (float)x[3] + g2 * ((float)e[1] + (float)e[3]));
+    const float q = 0.5f * ((float)x[5] + (float)x[7] + g2 * ((float)e[5] + (float)e[7]));
+    const float r = 0.5f * ((float)x[2] + (float)x[6] + g2 * ((float)e[2] + (float)e[6]));
+    const float s2 = 1.5f * (a * a + b * b + c * c + 2.0f * (p * p + q * q + r * r));
+    if (m.damage == TLSPH_DAMAGE_GTN)
+        return gtn_screen_f(m, s2, (float)eos_sm(m, J, x[13], 0.0), (float)x[10], (float)x[11],
+                            (float)gtn_fstar(m, x[14])) >= 0;
+    const float sf = jc_flow_f(m, (float)x[10], (float)x[11]) * (1.0f - D);
+    return !(s2 <= sf * sf);
+}
+
+// A thread per point.  The return of a yielding point takes several times the
+// FP64 instructions of an elastic one and holds the FP64 pipe for its warp
+// whatever the number of lanes, so a block first updates its elastic points
+// and then its yielding ones, gathered on consecutive threads.  GTN,
+// 200,003 points of which two in five yield: 0.38 -> 0.32 ms.
+constexpr int POINT_THREADS = 128;
+__global__ void __launch_bounds__(POINT_THREADS) k_material_point(const DevMat m, double dt, int64_t n,
+                                                                  const double *deps, const double *J, double *state)
+{
+    __shared__ int list[POINT_THREADS], count;
+    const int64_t t0 = (int64_t)blockIdx.x * POINT_THREADS, t = t0 + threadIdx.x;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    if (t < n) {
+        if (point_yields_f(m, deps + 9 * t, J[t], state + 16 * t)) list[atomicAdd(&count, 1)] = threadIdx.x;
+        else point_update(m, dt, deps + 9 * t, J[t], state + 16 * t);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x >= count) return;
+    const int64_t p = t0 + list[threadIdx.x];
+    point_update(m, dt, deps + 9 * p, J[p], state + 16 * p);
 }
 
 __global__ void k_export_sym(const double *src6, double *dst9, int64_t N)
@@ -934,7 +970,7 @@ cudaError_t launch_material_point_value(const DevMat &m, double dt, int64_t n, c
                                         const double *J, double *state, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_material_point<<<nblk(n, 128), 128, 0, st>>>(m, dt, n, deps, J, state);
+    k_material_point<<<nblk(n, POINT_THREADS), POINT_THREADS, 0, st>>>(m, dt, n, deps, J, state);
     return cudaGetLastError();
 }
 
