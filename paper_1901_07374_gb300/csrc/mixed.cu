@@ -1255,17 +1255,20 @@ __global__ void __launch_bounds__(128, 9) k_gather1_mixed_t4w(DevState s, MixCon
 //   12,000   70 | 42 / 33 / 39 / 47        64,200   97 | 98 / 121 / 156 / 197
 // Pass 1 alone still gains from two lanes up to 100,000 particles, with its
 // per-particle part in kernels of its own (Taylor cylinder of 60,000: 59 -> 53).
+// Launching each kernel while the one before finishes (`early`) takes the
+// first column to 14 (2048), 22 (5148) and 29 (12,000) and costs 11 % at 25,000.
 struct RowLanes {
     int pass1, pass2;   // lanes per row; 1: the plan's own kernels
     bool fused;         // pass 1 with the per-particle part in the same kernel
+    bool early;         // launched while the kernel before finishes (pdl_wait)
 };
 static RowLanes row_lanes(int64_t N)
 {
-    if (N < 4096) return { 16, 16, true };
-    if (N < 8192) return { 8, 8, true };
-    if (N < 20000) return { 4, 4, true };
-    if (N < 50000) return { 2, 2, true };
-    return { N < 100000 ? 2 : 1, 1, false };
+    if (N < 4096) return { 16, 16, true, true };
+    if (N < 8192) return { 8, 8, true, true };
+    if (N < 20000) return { 4, 4, true, true };
+    if (N < 50000) return { 2, 2, true, false };
+    return { N < 100000 ? 2 : 1, 1, false, false };
 }
 template <class F>
 static void with_lanes(int lanes, F &&f)
@@ -1292,6 +1295,7 @@ __global__ void __launch_bounds__(128) k_pass1_mixed_rows(DevState s, MixConst c
     __shared__ float sums[9][ROWS];
     const int sub = threadIdx.x % L, slot = threadIdx.x / L;
     const int64_t row0 = (int64_t)blockIdx.x * ROWS, i = row0 + slot;
+    pdl_wait();
     float m[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = 0.0f;
@@ -1308,6 +1312,7 @@ __global__ void __launch_bounds__(128) k_pass1_mixed_rows(DevState s, MixConst c
 #pragma unroll
         for (int k = 0; k < 9; ++k) sums[k][slot] = m[k];
     __syncthreads();
+    pdl_release();
     // this form leaves no queue behind: the other forms find it empty
     if (blockIdx.x == 0 && threadIdx.x == 0) s.slowq_n[0] = s.slowq_n[1] = 0u;
     if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
@@ -1323,6 +1328,7 @@ __global__ void __launch_bounds__(128) k_pass2_mixed_rows(DevState s, MixConst c
     __shared__ float sums[9][ROWS];
     const int sub = threadIdx.x % L, slot = threadIdx.x / L;
     const int64_t row0 = (int64_t)blockIdx.x * ROWS, i = row0 + slot;
+    pdl_wait();
     float m[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = 0.0f;
@@ -1333,6 +1339,7 @@ __global__ void __launch_bounds__(128) k_pass2_mixed_rows(DevState s, MixConst c
         if (sub == 0) sums[k][slot] = m[k];
     }
     __syncthreads();
+    pdl_release();
     if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = sums[k][threadIdx.x];
@@ -1632,8 +1639,8 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
     if (rows1) {
         with_lanes(rl.pass1, [&](auto lanes) {
             constexpr int L = decltype(lanes)::value;
-            if (fused1) k_pass1_mixed_rows<L, true><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
-            else k_pass1_mixed_rows<L, false><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+            launch_early(rl.early, fused1 ? k_pass1_mixed_rows<L, true> : k_pass1_mixed_rows<L, false>,
+                         nb(s.N, 128 / L), 128, st, s, c);
         });
         if (!fused1) k_epi1_mixed<<<nb(s.N, 128), 128, 0, st>>>(s, c);
     } else
@@ -1662,8 +1669,8 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
     if (v2 == 4 && rl.pass2 > 1) {
         with_lanes(rl.pass2, [&](auto lanes) {
             constexpr int L = decltype(lanes)::value;
-            if (hg) k_pass2_mixed_rows<true, L><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
-            else k_pass2_mixed_rows<false, L><<<nb(s.N, 128 / L), 128, 0, st>>>(s, c);
+            launch_early(rl.early, hg ? k_pass2_mixed_rows<true, L> : k_pass2_mixed_rows<false, L>, nb(s.N, 128 / L),
+                         128, st, s, c);
         });
     } else if (v2 == 1) {
         if (hg) k_pass2_mixed_t<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pair_id(DevState s, const int6
 template <int G>
 __global__ void __launch_bounds__(STEP_THREADS) k_pair_hourglass(DevState s, int ucur)
 {
+    pdl_wait();
     const int64_t i = ((int64_t)blockIdx.x * STEP_THREADS + threadIdx.x) / G;
     if (i >= s.N) return;
     const double *__restrict__ X = s.X;
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass1_fp64(DevState s, StepCon
     const double *__restrict__ X = s.X;
     const double *__restrict__ vh = s.vh;
     const bool tab = s.ptab != nullptr;
+    pdl_wait();
     double m[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = 0.0;
@@ -283,6 +285,7 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass1_fp64(DevState s, StepCon
         if (sub == 0) sums[k][slot] = t;
     }
     __syncthreads();
+    pdl_release();
     if (threadIdx.x >= ROWS || row0 + threadIdx.x >= s.N) return;
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = sums[k][threadIdx.x];
@@ -417,6 +420,7 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass2_fp64(DevState s, StepCon
     const double *__restrict__ Aa = s.A;
     const double *__restrict__ Fa = s.F;
     const bool tab = s.ptab != nullptr;
+    pdl_wait();
     double acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = 0.0;
@@ -485,6 +489,7 @@ __global__ void __launch_bounds__(STEP_THREADS) k_pass2_fp64(DevState s, StepCon
         if (sub == 0) sums[k][slot] = t;
     }
     __syncthreads();
+    pdl_release();
     const int64_t r = row0 + threadIdx.x;
     if (threadIdx.x >= ROWS || r >= s.N) return;
 #pragma unroll
@@ -929,23 +934,24 @@ cudaError_t launch_step_fp64(const DevState &s, const tlsph_config &cfg, int ucu
                              int64_t step_index, cudaStream_t st, cudaEvent_t *ev)
 {
     const StepConst c = make_const(cfg, ucur, dcur, step_index);
+    // launched while the kernel before finishes: 2048 particles 64.5 -> 58.9 us per step, 12,000 particles 164 -> 178
+    const bool early = s.N < 4096;
     if (ev) cudaEventRecord(ev[0], st);
     with_lanes(pass1_lanes(s.N), [&](auto lanes) {
         constexpr int G = decltype(lanes)::value;
-        k_pass1_fp64<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, c);
+        launch_early(early, k_pass1_fp64<G>, nblk(s.N, STEP_THREADS / G), STEP_THREADS, st, s, c);
     });
     if (ev) cudaEventRecord(ev[1], st);
     const bool hg = cfg.hg_alpha != 0.0;
     if (hg && s.ptab)
         with_lanes(hourglass_lanes(s.N), [&](auto lanes) {
             constexpr int G = decltype(lanes)::value;
-            k_pair_hourglass<G><<<nblk(s.N, STEP_THREADS / G), STEP_THREADS, 0, st>>>(s, ucur);
+            launch_early(early, k_pair_hourglass<G>, nblk(s.N, STEP_THREADS / G), STEP_THREADS, st, s, ucur);
         });
     with_lanes(row_lanes(s.N), [&](auto lanes) {
         constexpr int G = decltype(lanes)::value;
-        const unsigned grid = nblk(s.N, STEP_THREADS / G);
-        if (hg) k_pass2_fp64<G, true><<<grid, STEP_THREADS, 0, st>>>(s, c);
-        else k_pass2_fp64<G, false><<<grid, STEP_THREADS, 0, st>>>(s, c);
+        launch_early(early, hg ? k_pass2_fp64<G, true> : k_pass2_fp64<G, false>, nblk(s.N, STEP_THREADS / G),
+                     STEP_THREADS, st, s, c);
     });
     if (ev) cudaEventRecord(ev[2], st);
     return cudaGetLastError();

@@ -605,6 +605,33 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
     return status;
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// A kernel launched with `early` may become resident while the kernel before it
+// on the stream finishes (once each of that one's blocks has called
+// pdl_release or ended); its pdl_wait returns when every kernel before it has
+// finished and its writes are visible.  Both calls are no-ops in a kernel
+// launched without it.  Small grids only: blocks that arrive early are placed
+// around those still running, which unbalances a grid of several blocks per SM.
+// The release stands after the pair sums: at the start of the kernel it made
+// the 2048-particle steps slower (FP64 63.5 -> 79 us).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline void launch_early(bool early, void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);      // errors are read by cudaGetLastError
+}
+
 // ---------------------------------------------------------------- warp helpers
 __device__ __forceinline__ double warp_allsum(double x)
 {
