@@ -199,23 +199,48 @@ __device__ __forceinline__ float gap(float c, float lo, float w) { return fmaxf(
 // Threads take the particles in cell order, so the lanes of a warp search
 // nearly the same cells, and the candidates of a line of cells are consecutive
 // 16-byte records that carry their index: one load per candidate, shared by
-// the warp.  Bound by the latency of those loads and the few instructions per
-// candidate (about 261 candidates a particle).  On 209,827 particles the whole
-// of tlsph_neighbors_noalloc went from 5.5 ms (FP64 predicate on every
-// candidate, index and position fetched apart, one-block bounding box) to
-// 0.56 ms.
-__global__ void k_nbr(const double *X, int64_t N, GridArgs a, const int32_t *__restrict__ cell_start,
-                      const float4 *__restrict__ sorted, double rc2, int64_t *count, const int64_t *row_ptr,
-                      int32_t *out, Prefilter pf)
+// the warp.  A candidate too near the cutoff for FP32 goes to a list of its
+// thread, tested by the FP64 predicate after the search, all lanes together:
+// on an exact lattice 30 of a particle's candidates lie at the cutoff, and
+// tested where they are met they make nearly every turn of the loop wait for
+// the FP64 test of some lane (Taylor cylinder of 60,000: 386 us against 95).
+// Bound by the few instructions per candidate (about 261 a particle; lanes end
+// their lines at different turns, 20 of 32 active) and their load latency; 2 to
+// 8 threads per particle, dealt its lines of cells, were slower at 209,827
+// particles (0.71 to 1.6 ms for the whole service against 0.51).  The FP64
+// predicate on every candidate, index and position fetched apart, and a
+// one-block bounding box took 5.5 ms there.
+constexpr int NBR_THREADS = 128, NBR_BAND = 32;
+
+// the FP64 predicate on a thread's list: n with the neighbours found.  Not
+// inlined: predicated into the search's loop it holds the FP64 pipe for every
+// candidate.
+__device__ __noinline__ int test_band(const double *X, int64_t i, double rc2, const int *list, int count, int32_t *o,
+                                      int n)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int k = 0; k < count; ++k) {
+        const int j = list[k * NBR_THREADS];
+        if (!within(X + 3 * i, X + 3 * (int64_t)j, rc2)) continue;
+        if (o) o[n] = j;
+        ++n;
+    }
+    return n;
+}
+
+__global__ void __launch_bounds__(NBR_THREADS) k_nbr(const double *X, int64_t N, GridArgs a,
+                                                     const int32_t *__restrict__ cell_start,
+                                                     const float4 *__restrict__ sorted, double rc2, int64_t *count,
+                                                     const int64_t *row_ptr, int32_t *out, Prefilter pf)
+{
+    __shared__ int band[NBR_BAND][NBR_THREADS];
+    const int64_t t = (int64_t)blockIdx.x * NBR_THREADS + threadIdx.x;
     if (t >= N) return;
     const float4 fi = sorted[t];
     const int64_t i = __float_as_int(fi.w);
     int cx, cy, cz;
     cell_of(a, X + 3 * i, cx, cy, cz);
-    int n = 0;
     int32_t *o = out ? out + row_ptr[i] : nullptr;
+    int n = 0, nband = 0;
     const int R = a.reach;
     for (int z = max(cz - R, 0); z <= min(cz + R, a.nc2 - 1); ++z) {
         const float dz = gap(fi.z, fmaf((float)z, a.fcs, a.flo2), a.fcs);
@@ -232,20 +257,35 @@ __global__ void k_nbr(const double *X, int64_t N, GridArgs a, const int32_t *__r
             if (x0 > x1) continue;
             // cells x0..x1 of this (y, z) line are contiguous in the cell order
             const int b = cell_start[rowc + x0], e = cell_start[rowc + x1 + 1];
-            for (int k = b; k < e; ++k) {
-                const float4 fj = sorted[k];
-                const float dx = fj.x - fi.x, dy2 = fj.y - fi.y, dz3 = fj.z - fi.z;
-                const float r2f = dx * dx + dy2 * dy2 + dz3 * dz3;
-                if (r2f > pf.hi || k == t) continue;
-                const int j = __float_as_int(fj.w);
-                if (r2f >= pf.lo && !within(X + 3 * i, X + 3 * (int64_t)j, rc2)) continue;
-                if (o) o[n] = j;
-                ++n;
+            for (int k0 = b; k0 < e; k0 += 4) {     // four candidates in flight
+                float4 c[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[u] = sorted[min(k0 + u, e - 1)];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float ex = c[u].x - fi.x, ey = c[u].y - fi.y, ez = c[u].z - fi.z;
+                    const float r2f = ex * ex + ey * ey + ez * ez;
+                    const int j = __float_as_int(c[u].w);
+                    if (r2f > pf.hi || k0 + u >= e || j == (int)i) continue;
+                    if (r2f >= pf.lo) {
+                        band[nband++][threadIdx.x] = j;
+                        if (nband == NBR_BAND) {
+                            n = test_band(X, i, rc2, &band[0][threadIdx.x], nband, o, n);
+                            nband = 0;
+                        }
+                        continue;
+                    }
+                    if (o) o[n] = j;
+                    ++n;
+                }
             }
         }
     }
+    n = test_band(X, i, rc2, &band[0][threadIdx.x], nband, o, n);
     if (!o) count[i] = n;
 }
+
+static unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // Rows sorted ascending, one warp per row: a bitonic network over E elements
 // (E / 32 per lane, element e = k * 32 + lane, padded with INT_MAX); rows
@@ -321,8 +361,6 @@ __global__ void k_sort_rows(const int64_t *row_ptr, int32_t *col, int64_t N)
     }
 }
 
-static unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
-
 // prefilter thresholds for the grid's box: the FP32 positions are centred on
 // the box, so each coordinate carries at most delta = half extent x 2^-24;
 // |r2f - r2| <= 4 sqrt(3) rc delta + 4 sqrt(3) delta^2 + 4 2^-24 rc^2 for a
@@ -378,8 +416,8 @@ cudaError_t build_neighbors_count(const DevState &s, const CellGrid &g, const Sc
         return e;
     k_cell_scatter<<<blocks_for(s.N, 256), 256, 0, st>>>(s.X, s.N, a, pf, sc.cell_start, sc.slot, sc.sorted);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, row_ptr, nullptr, nullptr,
-                                                 pf);
+    k_nbr<<<blocks_for(s.N, NBR_THREADS), NBR_THREADS, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, row_ptr,
+                                                                nullptr, nullptr, pf);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(row_ptr + s.N, 0, sizeof(int64_t), st)) != cudaSuccess) return e;
     return scan_exclusive_i64(row_ptr, s.N + 1, sc.scan_tmp, st);
@@ -390,8 +428,9 @@ cudaError_t build_neighbors_fill(const DevState &s, const CellGrid &g, const Scr
 {
     const Prefilter pf = prefilter_for(g, rc2);
     const GridArgs a = clip_args(g, pf, rc2);
-    k_nbr<<<blocks_for(s.N, 128), 128, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, nullptr, row_ptr, col, pf);
-    cudaError_t e = cudaGetLastError();
+    k_nbr<<<blocks_for(s.N, NBR_THREADS), NBR_THREADS, 0, st>>>(s.X, s.N, a, sc.cell_start, sc.sorted, rc2, nullptr,
+                                                                row_ptr, col, pf);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_sort_rows<<<blocks_for(s.N * 32, 256), 256, 0, st>>>(row_ptr, col, s.N);
     return cudaGetLastError();
