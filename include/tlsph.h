@@ -271,12 +271,10 @@ int tlsph_destroy(tlsph_ctx *ctx);
  * does not fit; block size at most 128), plan[1] its block size, plan[2]
  * pass-2 form (0 warp
  * per 32 rows; 1 thread per row, two pairs in flight; 2 thread-per-row
- * gather + per-particle kernel; 3 thread per row, one pair in flight; 4 as
- * 1 with registers capped for six resident blocks; 5 as 3 with registers
- * capped for eight resident blocks; 6 as 1 capped for seven resident blocks;
- * 7 as 1 capped for five resident blocks; 8 as 7 with rows 0 and 1 of the
- * stress term formed by packed FP32x2 operations; block size at most 128 for
- * 4 to 8),
+ * gather + per-particle kernel; 3 thread per row, one pair in flight; 4, 7
+ * and 8 thread per row, eight slots a turn, registers capped for five resident
+ * blocks; 5 as 3 with registers capped for eight resident blocks; 6 as 1
+ * capped for seven resident blocks; block size at most 128 for 4 to 8),
  * plan[3] its block size (multiples of 32 up to 256).  On contexts of less
  * than 100,000 particles (pass 1) or 50,000 (pass 2) the pass-1 forms 4 and 5
  * and the pass-2 form 4 deal each row to 2 to 16 threads, in blocks of 128
@@ -362,9 +360,8 @@ const char *tlsph_batch_last_error(const tlsph_batch *b);
  * setting): shape[k] selects a variant for kernel kind
  * k = 0 (pass-1 gather), 1 (per-particle update), 2 (pass 2); a variant
  * fixes how many blocks of 128 threads the kernel's registers are capped for
- * and how many neighbour pairs a thread has in flight (and, for one pass-2
- * variant, packed FP32x2 stress rows as in pass-2 plan form 8; pass-1 variant
- * 4 reads each member's per-slot weight table as pass-1 plan form 5 does,
+ * and how many neighbour pairs a thread has in flight (pass-1 variant 4 reads
+ * each member's per-slot weight table as pass-1 plan form 5 does,
  * building the tables members lack: TLSPH_ERR_ARG for a member in a caller
  * arena, and a member whose table is released by its own tlsph_set_plan
  * stops tlsph_batch_step with TLSPH_ERR_STATE until tlsph_batch_set).  n must

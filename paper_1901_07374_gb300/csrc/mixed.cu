@@ -296,56 +296,97 @@ __global__ void k_ell_fill(const int64_t *row_ptr, const int32_t *col, int64_t N
     for (int k = 0; k < wv; ++k) o[32 * k + lane] = k < n ? col[b + k] : pad;
 }
 
+// one group of U slots of an aligned slice from slot k on: bits holds their
+// mask bits; CLAMP replaces an index outside the particle range (only ever a
+// masked slot) by alt
+template <int U, bool CLAMP, class Body>
+__device__ __forceinline__ void aligned_group(const int32_t *__restrict__ base, int k, uint32_t bits, int ii, int alt,
+                                              int N, Body &&body)
+{
+    int o[U];
+    // the table is 128-byte aligned and k a multiple of U: 8- or 16-byte loads
+    if constexpr (U >= 4) {
+#pragma unroll
+        for (int u = 0; u < U; u += 4) {
+            const int4 t = *reinterpret_cast<const int4 *>(base + k + u);
+            o[u] = t.x;
+            o[u + 1] = t.y;
+            o[u + 2] = t.z;
+            o[u + 3] = t.w;
+        }
+    } else if constexpr (U == 2) {
+        const int2 t = *reinterpret_cast<const int2 *>(base + k);
+        o[0] = t.x;
+        o[1] = t.y;
+    } else {
+        o[0] = base[k];
+    }
+    int j[U];
+    float w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const unsigned ju = (unsigned)ii + (unsigned)o[u];   // modular: a negative index wraps high
+        j[u] = (CLAMP && ju >= (unsigned)N) ? alt : (int)ju;
+        w[u] = (bits & (1u << u)) ? 0.0f : SLOT_PAD_Q;
+    }
+    body(j, w, k, std::integral_constant<int, U>());
+}
+
 // aligned slice: slots in groups of U, every L-th group from group `sub` on
-// (L lanes share a row); CLAMP replaces an index outside the particle range
-// (only ever a masked slot) by alt
-template <int U, bool CLAMP, int L, class Body>
+// (L lanes share a row); the last W mod U slots in groups of TU (L = 1)
+template <int U, bool CLAMP, int L, int TU, class Body>
 __device__ __forceinline__ void aligned_slots(const int32_t *__restrict__ base, int W, int lane, int ii, int alt,
                                               int N, int sub, Body &&body)
 {
     const int T = 32 * ((W + 31) / 32);
     const uint32_t *__restrict__ mk = reinterpret_cast<const uint32_t *>(base) + T + lane;
+    if constexpr (L > 1) {
+        for (int k = U * sub; k < W; k += U * L)
+            aligned_group<U, CLAMP>(base, k, mk[k & ~31] >> (k & 31), ii, alt, N, body);
+        return;
+    }
     uint32_t bits = 0;
-    for (int k = L > 1 ? U * sub : 0; k < W; k += U * L) {
-        if (L > 1) bits = mk[k & ~31] >> (k & 31);
-        else if ((k & 31) == 0) bits = mk[k];
-        int o[U];
-        // the table is 128-byte aligned and k a multiple of U: one 8- or 16-byte load for the group
-        if (U == 2) {
-            const int2 t = *reinterpret_cast<const int2 *>(base + k);
-            o[0] = t.x;
-            o[U - 1] = t.y;
-        } else if (U == 4) {
-            const int4 t = *reinterpret_cast<const int4 *>(base + k);
-            o[0] = t.x;
-            o[1 % U] = t.y;
-            o[2 % U] = t.z;
-            o[3 % U] = t.w;
-        } else {
-#pragma unroll
-            for (int u = 0; u < U; ++u) o[u] = base[k + u];
+    const int W0 = TU < U ? W - W % U : W;
+    int k = 0;
+    for (; k < W0; k += U) {
+        if ((k & 31) == 0) bits = mk[k];
+        aligned_group<U, CLAMP>(base, k, bits, ii, alt, N, body);
+        if constexpr (U < 32) bits >>= U;
+    }
+    if constexpr (TU < U) {
+        for (; k < W; k += TU) {
+            if ((k & 31) == 0) bits = mk[k];
+            aligned_group<TU, CLAMP>(base, k, bits, ii, alt, N, body);
+            bits >>= TU;
         }
-        int j[U];
-        float w[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const unsigned ju = (unsigned)ii + (unsigned)o[u];   // modular: a negative index wraps high
-            j[u] = (CLAMP && ju >= (unsigned)N) ? alt : (int)ju;
-            w[u] = (bits & (1u << u)) ? 0.0f : SLOT_PAD_Q;
-        }
-        if (L == 1) bits >>= U;
-        body(j, w, k);
     }
 }
 
-// Neighbour slots of row i in groups of U (U divides 32): body(j[U], qpad[U])
-// for each group, qpad = 0 for a neighbour and SLOT_PAD_Q for a padding slot
+// one group of U slots of an explicit slice of wv slots
+template <int U, class Body>
+__device__ __forceinline__ void explicit_group(const int32_t *__restrict__ cp, int k, int wv, int alt, Body &&body)
+{
+    int j[U];
+    float w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int kk = k + u;
+        const int jj = kk < wv ? cp[32 * kk] : ~alt;
+        j[u] = jj >= 0 ? jj : ~jj;
+        w[u] = jj >= 0 ? 0.0f : SLOT_PAD_Q;
+    }
+    body(j, w, k, std::integral_constant<int, U>());
+}
+
+// Neighbour slots of row i in groups of U (U divides 32), the last ones in
+// groups of TU: body(j[U], qpad[U], k, U) for each group, qpad = 0 for a
+// neighbour and SLOT_PAD_Q for a padding slot
 // (whose j is a valid particle other than i, so its terms are finite).  The
 // pair terms add qpad to the kernel argument q = r / h: a padding slot lands
 // outside the kernel's support (q >= 2), where W and W' are exactly zero, so
 // its terms vanish without a weight multiply.  With L > 1 the row's groups are
 // dealt to L lanes and this is the turn of lane `sub`.
-template <int U, int L = 1, class Body>
+template <int U, int L = 1, int TU = U, class Body>
 __device__ __forceinline__ void for_slots(const DevState &s, int64_t i, int sub, Body &&body)
 {
     const int64_t g = i >> 5;
@@ -355,22 +396,15 @@ __device__ __forceinline__ void for_slots(const DevState &s, int64_t i, int sub,
     const int alt = i == 0 ? 1 : (int)i - 1;
     if (wv < 0) {
         const int W = (~wv) & 0xffffff;
-        if ((~wv) >> 24) aligned_slots<U, true, L>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
-        else aligned_slots<U, false, L>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
+        if ((~wv) >> 24) aligned_slots<U, true, L, TU>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
+        else aligned_slots<U, false, L, TU>(base, W, lane, (int)i, alt, (int)s.N, sub, body);
     } else {
         const int32_t *__restrict__ cp = base + lane;
-        for (int k = L > 1 ? U * sub : 0; k < wv; k += U * L) {
-            int j[U];
-            float w[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int kk = k + u;
-                const int jj = kk < wv ? cp[32 * kk] : ~alt;
-                j[u] = jj >= 0 ? jj : ~jj;
-                w[u] = jj >= 0 ? 0.0f : SLOT_PAD_Q;
-            }
-            body(j, w, k);
-        }
+        const int W0 = TU < U ? wv - wv % U : wv;
+        int k = L > 1 ? U * sub : 0;
+        for (; k < W0; k += U * L) explicit_group<U>(cp, k, wv, alt, body);
+        if constexpr (TU < U)
+            for (; k < wv; k += TU) explicit_group<TU>(cp, k, wv, alt, body);
     }
 }
 
@@ -811,35 +845,33 @@ __device__ __forceinline__ void pair1(const MixConst &c, const int4 oi, const fl
 // thread per row over the sliced neighbour lists, U pairs in flight; with TAB
 // (four pairs in flight) the weights come from the per-slot table, one float4
 // per group of four slots, laid out [group][lane] within the slice
-template <int U, bool TAB = false, int L = 1>
+template <int U, bool TAB = false, int L = 1, int TU = U>
 __device__ __forceinline__ void gather1_row(const DevState &s, const MixConst &c, int64_t i, float *m, int sub = 0)
 {
     const int4 oi = s.xo[i];
     const float4 vi = s.r1[i];
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = 0.0f;
-    if constexpr (TAB) {
-        static_assert(U == 4, "the weight table holds groups of four slots");
-        const float4 *__restrict__ tb = s.w1t + s.w1t_off[i >> 5] + (i & 31);
-        for_slots<U, L>(s, i, sub, [&](const int *j, const float *, int k) {
-            int4 o[U];
-            float4 v[U];
+    const float4 *__restrict__ tb = TAB ? s.w1t + s.w1t_off[i >> 5] + (i & 31) : nullptr;
+    static_assert(!TAB || (U % 4 == 0 && TU % 4 == 0), "the weight table holds groups of four slots");
+    for_slots<U, L, TU>(s, i, sub, [&](const int *j, const float *w, int k, auto count) {
+        constexpr int n = decltype(count)::value;
+        int4 o[n];
+        float4 v[n];
 #pragma unroll
-            for (int u = 0; u < U; ++u) { o[u] = s.xo[j[u]]; v[u] = s.r1[j[u]]; }
-            const float4 t = tb[8 * k];      // group k / 4: float4 index 32 (k / 4) + lane
-            const float tw[4] = { t.x, t.y, t.z, t.w };
+        for (int u = 0; u < n; ++u) { o[u] = s.xo[j[u]]; v[u] = s.r1[j[u]]; }
+        if constexpr (TAB) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) pair1w(xdiff(o[u], oi), vi, v[u], tw[u % 4], m);
-        });
-        return;
-    }
-    for_slots<U, L>(s, i, sub, [&](const int *j, const float *w, int) {
-        int4 o[U];
-        float4 v[U];
+            for (int u = 0; u < n; u += 4) {
+                const float4 t = tb[8 * (k + u)];      // group k / 4: float4 index 32 (k / 4) + lane
+                const float tw[4] = { t.x, t.y, t.z, t.w };
 #pragma unroll
-        for (int u = 0; u < U; ++u) { o[u] = s.xo[j[u]]; v[u] = s.r1[j[u]]; }
+                for (int q = 0; q < 4; ++q) pair1w(xdiff(o[u + q], oi), vi, v[u + q], tw[q], m);
+            }
+        } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u) pair1(c, oi, vi, o[u], v[u], w[u], m);
+            for (int u = 0; u < n; ++u) pair1(c, oi, vi, o[u], v[u], w[u], m);
+        }
     });
 }
 
@@ -1046,11 +1078,9 @@ __device__ __forceinline__ Row2 load_row2(const DevState &s, const MixConst &c, 
 
 // Pair terms of row i with neighbour j (qpad: 0, or SLOT_PAD_Q for a padding
 // slot).  The row's own A and u are held negated, so the differences are sums.
-// With PK, rows 0 and 1 of (A_j - A_i) X_ij are formed together by packed
-// FP32x2 operations on the record's column pairs (same roundings as the
-// scalar form); the scalar form is the faster one on most lists, the packed
-// one on fully aligned lattice lists.
-template <bool HG, bool PK = false>
+// Packed FP32x2 operations on the record's column pairs were slower than this
+// form once a turn took eight slots (1.02M particles: 0.553 against 0.548 ms).
+template <bool HG>
 __device__ __forceinline__ void pair2(const DevState &s, const MixConst &c, const Row2 &w, int j, float qpad,
                                       float *acc)
 {
@@ -1067,18 +1097,8 @@ __device__ __forceinline__ void pair2(const DevState &s, const MixConst &c, cons
     const float gd = b2.y * g0;                    // V_j D_j W'/r
     acc[0] += gd * d.x; acc[1] += gd * d.y; acc[2] += gd * d.z;
     // (A_j - A_i) X_ij
-    float t0, t1;
-    if (PK) {
-        const float2 dx2 = make_float2(d.x, d.x), dy2 = make_float2(d.y, d.y), dz2 = make_float2(d.z, d.z);
-        const float2 t01 = __ffma2_rn(__fadd2_rn(make_float2(b1.x, b1.y), w.nA2), dz2,
-                                      __ffma2_rn(__fadd2_rn(make_float2(b0.z, b0.w), w.nA1), dy2,
-                                                 __fmul2_rn(__fadd2_rn(make_float2(b0.x, b0.y), w.nA0), dx2)));
-        t0 = t01.x;
-        t1 = t01.y;
-    } else {
-        t0 = (b0.x + w.nA0.x) * d.x + (b0.z + w.nA1.x) * d.y + (b1.x + w.nA2.x) * d.z;
-        t1 = (b0.y + w.nA0.y) * d.x + (b0.w + w.nA1.y) * d.y + (b1.y + w.nA2.y) * d.z;
-    }
+    const float t0 = (b0.x + w.nA0.x) * d.x + (b0.z + w.nA1.x) * d.y + (b1.x + w.nA2.x) * d.z;
+    const float t1 = (b0.y + w.nA0.y) * d.x + (b0.w + w.nA1.y) * d.y + (b1.y + w.nA2.y) * d.z;
     const float t2 = fmaf(b2.x + w.nA22, d.z, fmaf(b1.w + w.nA21, d.y, (b1.z + w.nA20) * d.x));
     acc[3] += g * t0; acc[4] += g * t1; acc[5] += g * t2;
     if (HG) {
@@ -1128,15 +1148,15 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
 }
 
 // pass-2 pair sums of row i over its slots, U pairs in flight
-template <bool HG, int U, bool PK = false, int L = 1>
+template <bool HG, int U, int L = 1, int TU = U>
 __device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c, int64_t i, float *acc, int sub = 0)
 {
     const Row2 w = load_row2<HG>(s, c, i);
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-    for_slots<U, L>(s, i, sub, [&](const int *j, const float *wm, int) {
+    for_slots<U, L, TU>(s, i, sub, [&](const int *j, const float *wm, int, auto count) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) pair2<HG, PK>(s, c, w, j[u], wm[u], acc);
+        for (int u = 0; u < decltype(count)::value; ++u) pair2<HG>(s, c, w, j[u], wm[u], acc);
     });
 }
 
@@ -1183,36 +1203,23 @@ __global__ void __launch_bounds__(128, 7) k_pass2_mixed_tc7(DevState s, MixConst
     epi2_mixed<HG>(s, c, i, acc);
 }
 
-// two pairs in flight, registers capped so that five blocks of 128 fit an SM
+// Eight slots a turn (the last of a row two a turn), registers capped so that
+// five blocks of 128 fit an SM: the slots' indices, masks and the loop cost
+// less per slot than at two a turn, and the loads of a turn's later slots move
+// under the arithmetic of its first.  Bound by instruction issue and the L1
+// data path together.  ms, two slots a turn capped for six blocks / five
+// blocks / five blocks with packed stress rows / this: 1.02M-particle bar
+// 0.569 / 0.563 / 0.557 / 0.548; notched bar of 455,958 0.332 / 0.297 / 0.312 /
+// 0.290; 128,000 0.116 / 0.096 / 0.104 / 0.095; Taylor cylinder of 60,000
+// 0.051 / 0.049 / 0.047 / 0.047.  Four slots a turn 0.556, sixteen 0.623, eight
+// to the end of the row 0.581 on the first.
 template <bool HG>
-__global__ void __launch_bounds__(128, 5) k_pass2_mixed_tc5(DevState s, MixConst c)
+__global__ void __launch_bounds__(128, 5) k_pass2_mixed_tc(DevState s, MixConst c)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.N) return;
     float acc[9];
-    gather2_row<HG, 2>(s, c, i, acc);
-    epi2_mixed<HG>(s, c, i, acc);
-}
-
-// as k_pass2_mixed_tc5 with the packed FP32x2 stress rows
-template <bool HG>
-__global__ void __launch_bounds__(128, 5) k_pass2_mixed_tc5p(DevState s, MixConst c)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= s.N) return;
-    float acc[9];
-    gather2_row<HG, 2, true>(s, c, i, acc);
-    epi2_mixed<HG>(s, c, i, acc);
-}
-
-// two pairs in flight, registers capped so that six blocks of 128 fit an SM
-template <bool HG>
-__global__ void __launch_bounds__(128, 6) k_pass2_mixed_tc(DevState s, MixConst c)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= s.N) return;
-    float acc[9];
-    gather2_row<HG, 2>(s, c, i, acc);
+    gather2_row<HG, 8, 1, 2>(s, c, i, acc);
     epi2_mixed<HG>(s, c, i, acc);
 }
 
@@ -1332,7 +1339,7 @@ __global__ void __launch_bounds__(128) k_pass2_mixed_rows(DevState s, MixConst c
     float m[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] = 0.0f;
-    if (i < s.N) gather2_row<HG, 2, false, L>(s, c, i, m, sub);
+    if (i < s.N) gather2_row<HG, 2, L>(s, c, i, m, sub);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         m[k] = lane_sum<L>(m[k]);
@@ -1503,7 +1510,7 @@ __global__ void __launch_bounds__(256) k_shape_mixed(DevState s, float inv_h, do
     float sm[9], cp[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) sm[k] = cp[k] = 0.0f;
-    for_slots<2>(s, i, 0, [&](const int *j, const float *w, int) {
+    for_slots<2>(s, i, 0, [&](const int *j, const float *w, int, auto) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const float3 d = xdiff(s.xo[j[u]], oi);
@@ -1583,7 +1590,7 @@ __global__ void __launch_bounds__(256) k_w1t_fill(DevState s, float inv_h)
         return;
     }
     const int4 oi = s.xo[i];
-    for_slots<4>(s, i, 0, [&](const int *j, const float *w, int k) {
+    for_slots<4>(s, i, 0, [&](const int *j, const float *w, int k, auto) {
         float t[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) t[u] = w1_weight(xdiff(s.xo[j[u]], oi), inv_h, w[u]);
@@ -1621,9 +1628,8 @@ int mixed_slow_grid()
 //           2 = thread-per-row gather + per-particle kernel;  3 = warp-per-32-rows gather + per-particle kernel;
 //           4 = as 2 with four pairs in flight per thread;  5 = as 4 with the weights W'/r from the per-slot table
 //   pass 2: 0 = warp per 32 rows;  1 = thread per row;  2 = thread-per-row gather + per-particle kernel;
-//           3 = thread per row, one pair in flight;  4 = thread per row, registers capped for 6 blocks of 128;
-//           5 = as 3 with registers capped for 8 blocks of 128;  6 = as 1 with registers capped for 7 blocks of 128;
-//           7 = as 1 with registers capped for 5 blocks of 128;  8 = as 7 with packed FP32x2 stress rows
+//           3 = thread per row, one pair in flight;  4, 7, 8 = thread per row, eight slots a turn;
+//           5 = as 3 with registers capped for 8 blocks of 128;  6 = as 1 with registers capped for 7 blocks of 128
 // block sizes are multiples of 32 up to 256 (128 for the fused warp forms and pass-2 forms 4 to 8).
 // Pass-1 forms 4 and 5 and pass-2 form 4 share a row between several lanes on small contexts (row_lanes).
 cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t st, cudaEvent_t *ev)
@@ -1678,18 +1684,12 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
     } else if (v2 == 3) {
         if (hg) k_pass2_mixed_t1<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_t1<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-    } else if (v2 == 4) {
-        if (hg) k_pass2_mixed_tc<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-        else k_pass2_mixed_tc<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
     } else if (v2 == 6) {
         if (hg) k_pass2_mixed_tc7<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_tc7<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-    } else if (v2 == 7) {
-        if (hg) k_pass2_mixed_tc5<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-        else k_pass2_mixed_tc5<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-    } else if (v2 == 8) {
-        if (hg) k_pass2_mixed_tc5p<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-        else k_pass2_mixed_tc5p<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
+    } else if (v2 == 4 || v2 == 7 || v2 == 8) {
+        if (hg) k_pass2_mixed_tc<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
+        else k_pass2_mixed_tc<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
     } else if (v2 == 5) {
         if (hg) k_pass2_mixed_t1c<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_t1c<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
@@ -1773,13 +1773,12 @@ __device__ __forceinline__ int batch_find(const int64_t *blk0, int n, int64_t w)
 // the compiler fuses).
 //   pass-1 gather:        (8, 4)  (6, 4)  (10, 4)  (8, 2)  (8, 4) with the members' per-slot weight tables
 //   per-particle update:  5  4  3
-//   pass 2:               (5, 2)  (6, 2)  (4, 2)  (8, 1)  (5, 2) with packed FP32x2 stress rows
+//   pass 2:               (5, 8)  (6, 2)  (4, 8)  (8, 1)  (5, 2); eight at a time end a row two at a time
 const int BATCH_VARIANTS[BATCH_KINDS] = { 5, 3, 5 };
 
-// ALT selects the alternative pair-term form of a kind: the per-slot weight
-// table in the pass-1 gather (members must hold one), the packed stress rows
-// in pass 2
-template <int KIND, bool HG, int MINB, int U, bool ALT = false>
+// TAB: the pass-1 gather reads the members' per-slot weight tables (members
+// must hold one)
+template <int KIND, bool HG, int MINB, int U, bool TAB = false>
 __global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchSlot *slots)
 {
     __shared__ uint64_t slot_words[(sizeof(BatchSlot) + 7) / 8];
@@ -1812,7 +1811,7 @@ __global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchS
             if (i < st.N) {
                 if constexpr (KIND == 0) {  // pass-1 gather
                     float mm[9];
-                    gather1_row<U, ALT>(st, c, i, mm);
+                    gather1_row<U, TAB>(st, c, i, mm);
 #pragma unroll
                     for (int k = 0; k < 9; ++k) st.fsum[k * st.N + i] = mm[k];
                 } else if (KIND == 1) {     // pass-1 per-particle update
@@ -1822,7 +1821,7 @@ __global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchS
                     epi1_mixed(st, c, i, mm);
                 } else {                    // pass 2
                     float acc[9];
-                    gather2_row<HG, U, ALT>(st, c, i, acc);
+                    gather2_row<HG, U, 1, U == 8 ? 2 : U>(st, c, i, acc);
                     epi2_mixed<HG>(st, c, i, acc);
                 }
             }
@@ -1907,10 +1906,10 @@ struct BatchKernel {
         } else {
             switch (v) {
             case 1: return k_batch<2, HG, 6, 2>;
-            case 2: return k_batch<2, HG, 4, 2>;
+            case 2: return k_batch<2, HG, 4, 8>;
             case 3: return k_batch<2, HG, 8, 1>;
-            case 4: return k_batch<2, HG, 5, 2, true>;
-            default: return k_batch<2, HG, 5, 2>;
+            case 4: return k_batch<2, HG, 5, 2>;
+            default: return k_batch<2, HG, 5, 8>;
             }
         }
     }
