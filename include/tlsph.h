@@ -272,9 +272,10 @@ int tlsph_destroy(tlsph_ctx *ctx);
  * pass-2 form (0 warp
  * per 32 rows; 1 thread per row, two pairs in flight; 2 thread-per-row
  * gather + per-particle kernel; 3 thread per row, one pair in flight; 4, 7
- * and 8 thread per row, eight slots a turn, registers capped for five resident
- * blocks; 5 as 3 with registers capped for eight resident blocks; 6 as 1
- * capped for seven resident blocks; block size at most 128 for 4 to 8),
+ * and 8 thread per row, eight slots a turn, in blocks of 320 from 400,000
+ * particles on whatever the plan's block size; 5 as 3 with registers capped
+ * for eight resident blocks; 6 as 1 capped for seven resident blocks; block
+ * size at most 128 for 4 to 8),
  * plan[3] its block size (multiples of 32 up to 256).  On contexts of less
  * than 100,000 particles (pass 1) or 50,000 (pass 2) the pass-1 forms 4 and 5
  * and the pass-2 form 4 deal each row to 2 to 16 threads, in blocks of 128

@@ -22,8 +22,8 @@ struct tlsph_batch {
     void *mem = nullptr;          // BatchHdr followed by capacity BatchSlots
     BatchHdr *hdr = nullptr;
     BatchSlot *slots = nullptr;
-    int64_t *blk0 = nullptr;        // capacity first work blocks (device), after the slots
-    std::vector<int64_t> blk0_host;
+    int64_t *blk0 = nullptr;        // 2 x capacity first work blocks (device), after the slots
+    std::vector<int64_t> blk0_host;  // the same, the second half at capacity
     std::vector<BatchSlot> host;
     std::vector<tlsph_ctx *> members;
     std::vector<int64_t> steps_at;  // each member's step count the table was built for
@@ -57,7 +57,7 @@ int tlsph_batch_create(int capacity, void *stream, tlsph_batch **out)
     if (!b) return TLSPH_ERR_NOMEM;
     b->capacity = capacity;
     b->stream = static_cast<cudaStream_t>(stream);
-    const size_t bytes = 256 + (size_t)capacity * sizeof(BatchSlot) + (size_t)capacity * sizeof(int64_t);
+    const size_t bytes = 256 + (size_t)capacity * sizeof(BatchSlot) + 2 * (size_t)capacity * sizeof(int64_t);
     if (cudaMalloc(&b->mem, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete b;
@@ -66,7 +66,7 @@ int tlsph_batch_create(int capacity, void *stream, tlsph_batch **out)
     b->hdr = static_cast<BatchHdr *>(b->mem);
     b->slots = reinterpret_cast<BatchSlot *>(static_cast<char *>(b->mem) + 256);
     b->blk0 = reinterpret_cast<int64_t *>(b->slots + capacity);
-    BatchHdr h{ 0, 0, b->blk0 };
+    BatchHdr h{ 0, { 0, 0 }, { b->blk0, b->blk0 + capacity } };
     if (cudaMemcpy(b->hdr, &h, sizeof h, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->start, cudaEventDisableTiming) != cudaSuccess ||
@@ -122,21 +122,23 @@ int tlsph_batch_set(tlsph_batch *b, tlsph_ctx *const *ctxs, int n)
     b->host.resize(n);
     b->members.assign(ctxs, ctxs + n);
     b->steps_at.resize(n);
-    int64_t blk = 0;
-    b->blk0_host.resize(n);
+    int64_t blk[2] = { 0, 0 };
+    const int rows[2] = { 128, BATCH_WIDE };
+    b->blk0_host.assign(2 * (size_t)b->capacity, 0);
     for (int k = 0; k < n; ++k) {
         b->host[k] = make_batch_slot(*ctxs[k]);
-        b->host[k].blk0 = blk;
-        b->blk0_host[k] = blk;
-        blk += (ctxs[k]->N + 127) / 128;
+        for (int w = 0; w < 2; ++w) {
+            b->host[k].blk0[w] = b->blk0_host[(size_t)w * b->capacity + k] = blk[w];
+            blk[w] += (ctxs[k]->N + rows[w] - 1) / rows[w];
+        }
         b->steps_at[k] = ctxs[k]->steps;
     }
-    BatchHdr h{ n, blk, b->blk0 };
+    BatchHdr h{ n, { blk[0], blk[1] }, { b->blk0, b->blk0 + b->capacity } };
     e = cudaStreamSynchronize(b->own);
     if (e == cudaSuccess && n > 0)
         e = cudaMemcpyAsync(b->slots, b->host.data(), (size_t)n * sizeof(BatchSlot), cudaMemcpyHostToDevice, b->own);
     if (e == cudaSuccess && n > 0)
-        e = cudaMemcpyAsync(b->blk0, b->blk0_host.data(), (size_t)n * sizeof(int64_t), cudaMemcpyHostToDevice, b->own);
+        e = cudaMemcpyAsync(b->blk0, b->blk0_host.data(), b->blk0_host.size() * sizeof(int64_t), cudaMemcpyHostToDevice, b->own);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->hdr, &h, sizeof h, cudaMemcpyHostToDevice, b->own);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->own);
     if (e != cudaSuccess) return batch_fail(b, TLSPH_ERR_CUDA, std::string("table upload: ") + cudaGetErrorString(e));

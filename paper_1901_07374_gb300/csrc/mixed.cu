@@ -49,6 +49,8 @@ namespace tlsph {
 
 static constexpr int MIX_THREADS = 128;
 
+static unsigned nb(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
+
 static MixConst make_mix_const(const tlsph_ctx &ctx, int64_t step_index)
 {
     MixConst c;
@@ -652,7 +654,7 @@ __device__ __forceinline__ void epi1_mixed(const DevState &s, const MixConst &c,
     }
     float Li[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Li[k] = s.linv32[9 * i + k];
+    for (int k = 0; k < 9; ++k) Li[k] = s.linv32[k * N + i];
     // dF = dt Fdot (Fdot = M L^{-1}, Sec. 3.1); F^{n+1} = F^n + dF compensated
     float dF[9];
 #pragma unroll
@@ -748,7 +750,7 @@ __device__ __forceinline__ void epi1_slow(const DevState &s, const MixConst &c, 
     for (int k = 0; k < 9; ++k) {
         Fh[k] = s.Fh[k * N + i];
         Fl[k] = s.Fl[k * N + i];
-        Li[k] = s.linv32[9 * i + k];
+        Li[k] = s.linv32[k * N + i];
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) sgn[k] = s.sigf[k * N + i];
@@ -1080,12 +1082,14 @@ __device__ __forceinline__ Row2 load_row2(const DevState &s, const MixConst &c, 
 // slot).  The row's own A and u are held negated, so the differences are sums.
 // Packed FP32x2 operations on the record's column pairs were slower than this
 // form once a turn took eight slots (1.02M particles: 0.553 against 0.548 ms).
-template <bool HG>
+// IDX32 forms the record's index in 32 bits: 6 N records, N under 7e8, which a
+// mixed context's more than 700 bytes per particle imply on a device of 288 GB.
+template <bool HG, bool IDX32>
 __device__ __forceinline__ void pair2(const DevState &s, const MixConst &c, const Row2 &w, int j, float qpad,
                                       float *acc)
 {
-    const int4 oj = s.xo[j];
-    const float4 *rj = s.r2 + r2_tile(j);
+    const int4 oj = s.xo[IDX32 ? (int64_t)(unsigned)j : (int64_t)j];
+    const float4 *rj = s.r2 + (IDX32 ? (int64_t)((unsigned)j + ((unsigned)j >> 5) * (6u * 32u - 32u)) : r2_tile(j));
     const float4 b0 = rj[0], b1 = rj[R2_STRIDE], b2 = rj[2 * R2_STRIDE];
     const float3 d = xdiff(oj, w.o);
     const float r2v = d.x * d.x + d.y * d.y + d.z * d.z;
@@ -1135,7 +1139,7 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
         float acc[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-        for (int64_t p = p0 + lane; p < p1; p += 32) pair2<HG>(s, c, w, s.col[p], 0.0f, acc);
+        for (int64_t p = p0 + lane; p < p1; p += 32) pair2<HG, false>(s, c, w, s.col[p], 0.0f, acc);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             if (!HG && k >= 6) continue;
@@ -1148,7 +1152,7 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
 }
 
 // pass-2 pair sums of row i over its slots, U pairs in flight
-template <bool HG, int U, int L = 1, int TU = U>
+template <bool HG, int U, int L = 1, int TU = U, bool IDX32 = false>
 __device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c, int64_t i, float *acc, int sub = 0)
 {
     const Row2 w = load_row2<HG>(s, c, i);
@@ -1156,7 +1160,7 @@ __device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
     for_slots<U, L, TU>(s, i, sub, [&](const int *j, const float *wm, int, auto count) {
 #pragma unroll
-        for (int u = 0; u < decltype(count)::value; ++u) pair2<HG>(s, c, w, j[u], wm[u], acc);
+        for (int u = 0; u < decltype(count)::value; ++u) pair2<HG, IDX32>(s, c, w, j[u], wm[u], acc);
     });
 }
 
@@ -1203,27 +1207,45 @@ __global__ void __launch_bounds__(128, 7) k_pass2_mixed_tc7(DevState s, MixConst
     epi2_mixed<HG>(s, c, i, acc);
 }
 
-// Eight slots a turn (the last of a row two a turn), registers capped so that
-// five blocks of 128 fit an SM: the slots' indices, masks and the loop cost
-// less per slot than at two a turn, and the loads of a turn's later slots move
-// under the arithmetic of its first.  Bound by instruction issue and the L1
-// data path together.  ms, two slots a turn capped for six blocks / five
-// blocks / five blocks with packed stress rows / this: 1.02M-particle bar
-// 0.569 / 0.563 / 0.557 / 0.548; notched bar of 455,958 0.332 / 0.297 / 0.312 /
-// 0.290; 128,000 0.116 / 0.096 / 0.104 / 0.095; Taylor cylinder of 60,000
-// 0.051 / 0.049 / 0.047 / 0.047.  Four slots a turn 0.556, sixteen 0.623, eight
-// to the end of the row 0.581 on the first.
-template <bool HG>
-__global__ void __launch_bounds__(128, 5) k_pass2_mixed_tc(DevState s, MixConst c)
+// Eight slots a turn: the slots' indices, masks and the loop cost less per slot
+// than at two a turn, and the loads of a turn's later slots move under the
+// arithmetic of its first.  Bound by the record loads' latency under 20 warps
+// per SM, with the issue slots and the L1 data path two thirds busy each.
+// Blocks of 320 rows, two to an SM, on large contexts: the warps of a block
+// walk their rows in step, so a wider block meets more of its neighbours'
+// records in L1; blocks of 128, five to an SM, below 400,000 particles, where a
+// few waves of wide blocks leave SMs idle.  ms, two slots a turn in blocks of
+// 128 (registers capped for six / five to an SM) / eight in blocks of 128 / 320:
+//   1.02M-particle bar   0.569 / 0.563   0.549   0.529
+//   Taylor 500,000       0.311 / 0.293   0.292   0.274
+//   notched bar 455,958  0.332 / 0.297   0.291   0.285
+//   256,000              0.168 / 0.157   0.156   0.159
+//   160,000 (Taylor)                     0.102   0.107
+//   60,000 (Taylor)      0.051 / 0.049   0.048   0.060
+// On the first in blocks of 320: four slots a turn 0.553, sixteen 0.559, a
+// row's last slots two a turn 0.535 and 64-bit record indices 0.540 (in blocks
+// of 128 these two are the better ones, 0.549 against 0.555); blocks of 160 /
+// 384 / 640 0.538 / 0.545 / 0.586; packed FP32x2 stress rows 0.553 in blocks of 128.
+constexpr int64_t PASS2_WIDE_FROM = 400000;
+template <bool HG, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 320 : 128, WIDE ? 2 : 5) k_pass2_mixed_tc(DevState s, MixConst c)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.N) return;
     float acc[9];
-    gather2_row<HG, 8, 1, 2>(s, c, i, acc);
+    gather2_row<HG, 8, 1, WIDE ? 1 : 2, WIDE>(s, c, i, acc);
     epi2_mixed<HG>(s, c, i, acc);
 }
 
-__global__ void __launch_bounds__(256) k_gather1_mixed_t4(DevState s, MixConst c)
+template <bool HG>
+static void launch_pass2_tc(const DevState &s, const MixConst &c, int block, cudaStream_t st)
+{
+    if (s.N >= PASS2_WIDE_FROM) k_pass2_mixed_tc<HG, true><<<nb(s.N, 320), 320, 0, st>>>(s, c);
+    else k_pass2_mixed_tc<HG, false><<<nb(s.N, block), block, 0, st>>>(s, c);
+}
+
+// registers capped for eight blocks of 128 to an SM: 1.02M particles 0.336 -> 0.326 ms with the update
+__global__ void __launch_bounds__(256, 4) k_gather1_mixed_t4(DevState s, MixConst c)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.N) return;
@@ -1395,7 +1417,7 @@ __global__ void k_mixed_static(DevState s, const double *S0)
     if (i >= s.N) return;
     s.s0[i] = make_float4((float)S0[3 * i], (float)S0[3 * i + 1], (float)S0[3 * i + 2], 0.0f);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) s.linv32[9 * i + k] = (float)s.Linv[9 * i + k];
+    for (int k = 0; k < 9; ++k) s.linv32[k * s.N + i] = (float)s.Linv[9 * i + k];
 }
 
 // pass-1 record from the FP64 half-step velocity and D^n
@@ -1464,8 +1486,6 @@ static int mixed_field_bits(int field)
     default: return 0;
     }
 }
-
-static unsigned nb(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 cudaError_t mixed_import(const tlsph_ctx &ctx, int field, cudaStream_t st)
 {
@@ -1688,8 +1708,8 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
         if (hg) k_pass2_mixed_tc7<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_tc7<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
     } else if (v2 == 4 || v2 == 7 || v2 == 8) {
-        if (hg) k_pass2_mixed_tc<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
-        else k_pass2_mixed_tc<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
+        if (hg) launch_pass2_tc<true>(s, c, b2, st);
+        else launch_pass2_tc<false>(s, c, b2, st);
     } else if (v2 == 5) {
         if (hg) k_pass2_mixed_t1c<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_t1c<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
@@ -1773,20 +1793,21 @@ __device__ __forceinline__ int batch_find(const int64_t *blk0, int n, int64_t w)
 // the compiler fuses).
 //   pass-1 gather:        (8, 4)  (6, 4)  (10, 4)  (8, 2)  (8, 4) with the members' per-slot weight tables
 //   per-particle update:  5  4  3
-//   pass 2:               (5, 8)  (6, 2)  (4, 8)  (8, 1)  (5, 2); eight at a time end a row two at a time
+//   pass 2:               (2 blocks of 320, 8)  (6, 2)  (5, 8)  (8, 1)  (5, 2)
 const int BATCH_VARIANTS[BATCH_KINDS] = { 5, 3, 5 };
 
 // TAB: the pass-1 gather reads the members' per-slot weight tables (members
 // must hold one)
-template <int KIND, bool HG, int MINB, int U, bool TAB = false>
-__global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchSlot *slots)
+template <int KIND, bool HG, int MINB, int U, bool TAB = false, int BLOCK = 128>
+__global__ void __launch_bounds__(BLOCK, MINB) k_batch(BatchHdr *hdr, const BatchSlot *slots)
 {
     __shared__ uint64_t slot_words[(sizeof(BatchSlot) + 7) / 8];
     __shared__ int64_t grab;
     const BatchSlot &sl = *reinterpret_cast<const BatchSlot *>(slot_words);
+    constexpr int WB = BLOCK == BATCH_WIDE ? 1 : 0;
     const int nspec = hdr->nspec;
-    const int64_t total = hdr->total_blk;
-    const int64_t *blk0 = hdr->blk0;
+    const int64_t total = hdr->total_blk[WB];
+    const int64_t *blk0 = hdr->blk0[WB];
     int cur = -1;
     // the first chunk is the block's own (blocks without one leave at once, touching no counter);
     // later chunks come from the counter, after the grid's first chunks
@@ -1807,7 +1828,7 @@ __global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchS
             }
             const DevState &st = sl.s;
             const MixConst &c = sl.c;
-            const int64_t i = (w - sl.blk0) * blockDim.x + threadIdx.x;
+            const int64_t i = (w - sl.blk0[WB]) * BLOCK + threadIdx.x;
             if (i < st.N) {
                 if constexpr (KIND == 0) {  // pass-1 gather
                     float mm[9];
@@ -1821,7 +1842,7 @@ __global__ void __launch_bounds__(128, MINB) k_batch(BatchHdr *hdr, const BatchS
                     epi1_mixed(st, c, i, mm);
                 } else {                    // pass 2
                     float acc[9];
-                    gather2_row<HG, U, 1, U == 8 ? 2 : U>(st, c, i, acc);
+                    gather2_row<HG, U, 1, U == 8 ? (WB ? 1 : 2) : U, WB == 1>(st, c, i, acc);
                     epi2_mixed<HG>(st, c, i, acc);
                 }
             }
@@ -1878,7 +1899,7 @@ BatchSlot make_batch_slot(const tlsph_ctx &ctx)
     BatchSlot b;
     b.s = ctx.s;
     b.c = make_mix_const(ctx, ctx.steps);
-    b.blk0 = 0;
+    b.blk0[0] = b.blk0[1] = 0;
     return b;
 }
 
@@ -1887,6 +1908,7 @@ BatchSlot make_batch_slot(const tlsph_ctx &ctx)
 template <int KIND, bool HG>
 struct BatchKernel {
     using fn = void (*)(BatchHdr *, const BatchSlot *);
+    static int block(int v) { return KIND == 2 && v == 0 ? BATCH_WIDE : 128; }
     static fn get(int v)
     {
         if (KIND == 0) {
@@ -1906,10 +1928,10 @@ struct BatchKernel {
         } else {
             switch (v) {
             case 1: return k_batch<2, HG, 6, 2>;
-            case 2: return k_batch<2, HG, 4, 8>;
+            case 2: return k_batch<2, HG, 5, 8>;
             case 3: return k_batch<2, HG, 8, 1>;
             case 4: return k_batch<2, HG, 5, 2>;
-            default: return k_batch<2, HG, 5, 8>;
+            default: return k_batch<2, HG, 2, 8, false, BATCH_WIDE>;
             }
         }
     }
@@ -1918,10 +1940,10 @@ struct BatchKernel {
 template <bool HG>
 static void batch_kernels(BatchHdr *hdr, BatchSlot *slots, const int *shape, const int *grid, cudaStream_t st)
 {
-    BatchKernel<0, HG>::get(shape[0])<<<grid[0], 128, 0, st>>>(hdr, slots);
-    BatchKernel<1, HG>::get(shape[1])<<<grid[1], 128, 0, st>>>(hdr, slots);
+    BatchKernel<0, HG>::get(shape[0])<<<grid[0], BatchKernel<0, HG>::block(shape[0]), 0, st>>>(hdr, slots);
+    BatchKernel<1, HG>::get(shape[1])<<<grid[1], BatchKernel<1, HG>::block(shape[1]), 0, st>>>(hdr, slots);
     k_batch_slow<<<grid[3], 128, 0, st>>>(hdr, slots);
-    BatchKernel<2, HG>::get(shape[2])<<<grid[2], 128, 0, st>>>(hdr, slots);
+    BatchKernel<2, HG>::get(shape[2])<<<grid[2], BatchKernel<2, HG>::block(shape[2]), 0, st>>>(hdr, slots);
 }
 
 cudaError_t launch_batch_step(BatchHdr *hdr, BatchSlot *slots, int nspec, bool hg, const int *shape, const int *grid,
@@ -1936,9 +1958,12 @@ cudaError_t launch_batch_step(BatchHdr *hdr, BatchSlot *slots, int nspec, bool h
 template <bool HG>
 static void batch_occupancy(const int *shape, int *per)
 {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], BatchKernel<0, HG>::get(shape[0]), 128, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[1], BatchKernel<1, HG>::get(shape[1]), 128, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[2], BatchKernel<2, HG>::get(shape[2]), 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], BatchKernel<0, HG>::get(shape[0]),
+                                                  BatchKernel<0, HG>::block(shape[0]), 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[1], BatchKernel<1, HG>::get(shape[1]),
+                                                  BatchKernel<1, HG>::block(shape[1]), 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[2], BatchKernel<2, HG>::get(shape[2]),
+                                                  BatchKernel<2, HG>::block(shape[2]), 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[3], k_batch_slow, 128, 0);
 }
 

@@ -76,7 +76,7 @@ struct DevState {
     // mixed-precision records (null in the FP64 path)
     int4 *xo;               // N   {fixed-point position x, y, z (FixPack), 0}
     float4 *s0;             // N   {sum_j V_j W'(r)/r (X_j - X_i), 0}  (static, FP64-accurate)
-    float *linv32;          // N*9 L^{-1} rounded
+    float *linv32;          // 9 x N L^{-1} rounded, SoA by component
     float4 *r1;             // N   pass-1 gather record {v^{n+1/2} - vref, V (1 - D)}
     float4 *r2;             // pass-2 gather record: 6 float4 per particle in tiles of 32 particles (r2_tile)
     float *fsum;            // 9 x N pass-1 pair sums (split launch plans)
@@ -282,16 +282,18 @@ struct MixConst {
     int wall;
 };
 
+// rows of a work block of the wide pass-2 variants
+constexpr int BATCH_WIDE = 320;
 // one context in a batch table (device memory)
 struct BatchSlot {
     DevState s;
     MixConst c;
-    int64_t blk0;      // first work block of this context
+    int64_t blk0[2];   // first work block of this context, in blocks of 128 and of BATCH_WIDE rows
 };
 struct BatchHdr {
     int nspec;
-    int64_t total_blk;
-    const int64_t *blk0;    // nspec first work blocks, ascending (device, after the slots)
+    int64_t total_blk[2];   // in blocks of 128 and of BATCH_WIDE rows
+    const int64_t *blk0[2]; // nspec first work blocks, ascending (device, after the slots)
     unsigned long long next[3];   // work-block counters of the three persistent kernels (zero between steps)
 };
 BatchSlot make_batch_slot(const tlsph_ctx &ctx);

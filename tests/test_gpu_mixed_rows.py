@@ -1,4 +1,4 @@
-"""The mixed path's row kernels for small contexts (a row dealt to 2 to 16
+"""The mixed path's row kernels for small contexts and the wide blocks of large ones (a row dealt to 2 to 16
 lanes, pass 1 with its FP64 updates in one kernel) at particle counts on
 either side of each rule, on aligned and explicit slices, elastic and in
 plastic flow, with and without the hourglass term: the default plan against a
@@ -16,7 +16,7 @@ from paper_1901_07374_gb300 import tlsph
 pytestmark = pytest.mark.gpu
 
 FIELDS = ("U", "V", "F", "SIGMA")
-SIZES = [31, 33, 4095, 4097, 8191, 8193, 19999, 20001, 49999, 50001, 99999, 100001]
+SIZES = [31, 33, 4095, 4097, 8191, 8193, 19999, 20001, 49999, 50001, 99999, 100001, 399999, 400001]
 
 
 def _bar(n, hg=10.0, shuffle=False, flow=True):
