@@ -387,6 +387,7 @@ DevMat make_dev_mat(const tlsph_material &m)
     d.inv_sN = m.sN > 0.0 ? 1.0 / m.sN : 0.0;
     double c = 1.0;
     for (int k = 0; k < 11; ++k) d.binom[k] = c *= (m.n - k) / (k + 1);
+    d.binom_r = m.n <= 2.0 ? 0.03125 : 0.0;
     d.fstar_slope = (m.fF > m.fc) ? (1.0 / m.q1 - m.fc) / (m.fF - m.fc) : 0.0;
     d.Kf = (float)d.K; d.Gf = (float)d.G; d.Af = (float)d.A; d.Bf = (float)d.B; d.nf = (float)d.n;
     d.Cf = (float)d.C; d.inv_epsdot0f = (float)d.inv_epsdot0; d.rho0c02f = (float)d.rho0c02;

@@ -163,11 +163,22 @@ __device__ __forceinline__ double rcp_fp64(double x)
     return fma(r, fma(e, e, e), r);
 }
 
+// sqrt(x) and its reciprocal for x below the range of the hardware's approximation
+static __device__ __noinline__ double2 sqrt_small(double x)
+{
+    const double s = sqrt(x);
+    return make_double2(s, 1.0 / s);
+}
 // sqrt(x) and 1 / sqrt(x) for x > 0: the hardware's approximation of the
 // reciprocal root refined by one step of Householder's third-order iteration,
 // r (1 + e / 2 + 3 e^2 / 8) with e = 1 - x r^2
 __device__ __forceinline__ double sqrt_fp64(double x, double &rinv)
 {
+    if (__double2hiint(x) < 0x03000000) {       // below 1e-290, where the approximation flushes its argument
+        const double2 s = sqrt_small(x);
+        rinv = s.y;
+        return s.x;
+    }
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r * r, 1.0);
@@ -182,6 +193,15 @@ __device__ __forceinline__ double div_fp64(double a, double b, double ib)
 {
     const double q = a * ib;
     return fma(ib, fma(-q, b, a), q);
+}
+
+// a / b, with the quotient's own division for b outside the range of the
+// reciprocal's approximation (0: a fully damaged particle's modulus)
+static __device__ __noinline__ double div_small(double a, double b) { return a / b; }
+__device__ __forceinline__ double quot_fp64(double a, double b)
+{
+    if (__double2hiint(b) < 0x03000000) return div_small(a, b);
+    return div_fp64(a, b, rcp_fp64(b));
 }
 
 // Rotation factor of the polar decomposition F = R U by Newton's iteration
@@ -447,7 +467,7 @@ __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const d
         x += d;
     }
     if (!conv) { status |= TLSPH_ST_NEWTON_CAP; shx = sinh(a1 * x); }
-    const double kf = fma(1.5 * m.q1 * m.q2 * f * tri, shx, x) * rcp_fp64(3.0 * m.G * omD * (1.0 - f));
+    const double kf = quot_fp64(fma(1.5 * m.q1 * m.q2 * f * tri, shx, x), 3.0 * m.G * omD * (1.0 - f));
     // matrix strain increment: root of g(de) = de - (seq - x sigma_f(ep + de)) kf
     const double ep0 = s.ep;
     const double xrk = x * rate * kf;
@@ -457,11 +477,11 @@ __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const d
     conv = false;
     const float ds = de > 0.0 ? gtn_de_seed32((float)ep0, (float)(h0 - m.A), (float)m.B, (float)m.n, (float)de, (float)xrk)
                               : -1.0f;
-    if (ds > 0.0f && ep0 > 0.0) {
+    if (ds > 0.0f && ep0 > 0.0 && m.binom_r > 0.0) {
         const double dx = (double)ds, H0 = h0 - m.A, ep = ep0 + dx, ie = rcp_fp64(ep);
         const double r = dx * rcp_fp64(ep0);
         double H;
-        if (r < 0.03125) {              // (1 + r)^n - 1 to r^11, the next term below 1e-18
+        if (r < m.binom_r) {            // (1 + r)^n - 1 to r^11, the next term below 1e-18
             double sum = m.binom[10];
 #pragma unroll
             for (int k = 9; k >= 0; --k) sum = fma(sum, r, m.binom[k]);
@@ -563,8 +583,7 @@ __device__ __forceinline__ uint32_t material_update(const DevMat &m, double dt, 
         } else {
             double iseq;
             const double seq = sqrt_fp64(s2, iseq);
-            const double g3 = 3.0 * m.G * omD;
-            dep = div_fp64(seq - sf, g3, rcp_fp64(g3));
+            dep = quot_fp64(seq - sf, 3.0 * m.G * omD);      // infinite at D = 1
             const double sc = div_fp64(sf, seq, iseq);
             seq1 = sf;
 #pragma unroll

@@ -26,6 +26,7 @@ struct DevMat {
     double nucl_coef;    // fN / (sN sqrt(2 pi))
     double inv_sN;
     double binom[11];    // binomial coefficients (n over k), k = 1 .. 11, of the hardening exponent
+    double binom_r;      // largest r the series of (1 + r)^n is used for: 1/32; 0 for n > 2 (its terms fall off too slowly)
     double fstar_slope;  // (1/q1 - fc) / (fF - fc)
     double g0rho0;       // Gamma0 rho0 (energy term of the Mie-Grueneisen EOS)
     double inv_rho0;
