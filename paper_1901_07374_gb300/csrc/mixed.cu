@@ -798,13 +798,23 @@ __device__ __forceinline__ void epi1_slow(const DevState &s, const MixConst &c, 
                 mat.inv_rho0f, Vf, u0, u1, u2, st);
 }
 
+// First slot of the FP64-update queue of a thread of a persistent grid: the
+// grid's warps take the queue 32 slots at a time in the order (warp of the
+// block, block), so that a short queue spreads over the SMs.  Bound by the SM's
+// FP64 pipe (an instruction of any warp holds it for 16 cycles): with the slots
+// dealt block by block a queue of a few thousand particles kept four warps on
+// each of a few dozen SMs.
+__device__ __forceinline__ uint32_t slow_slot()
+{
+    return ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u);
+}
+
 // persistent grid over the step's queue of FP64 updates; clears the queue
 // counter of the next step (the two counters alternate with the step parity)
 __global__ void __launch_bounds__(128) k_epi1_slow(DevState s, MixConst c)
 {
     const uint32_t n = s.slowq_n[c.step_index & 1];
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
-        epi1_slow(s, c, s.slowq[q]);
+    for (uint32_t q = slow_slot(); q < n; q += gridDim.x * blockDim.x) epi1_slow(s, c, s.slowq[q]);
     if (blockIdx.x == 0 && threadIdx.x == 0) s.slowq_n[(c.step_index + 1) & 1] = 0u;
 }
 
@@ -1864,7 +1874,8 @@ __global__ void __launch_bounds__(128) k_batch_slow(const BatchHdr *hdr, BatchSl
 {
     __shared__ uint32_t cnt[1024];
     const int nspec = hdr->nspec;
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const uint32_t t = slow_slot(), stride = gridDim.x * blockDim.x;
+    uint32_t first = t;         // this thread's first slot in the member's queue, as if the queues stood in a row
     for (int m0 = 0; m0 < nspec; m0 += 1024) {
         const int mn = min(1024, nspec - m0);
         for (int k = threadIdx.x; k < mn; k += blockDim.x) {
@@ -1876,7 +1887,9 @@ __global__ void __launch_bounds__(128) k_batch_slow(const BatchHdr *hdr, BatchSl
             const uint32_t n = cnt[k];
             if (n == 0) continue;
             const BatchSlot &sl = slots[m0 + k];
-            for (uint32_t q = t; q < n; q += stride) epi1_slow(sl.s, sl.c, sl.s.slowq[q]);
+            uint32_t q = first;
+            for (; q < n; q += stride) epi1_slow(sl.s, sl.c, sl.s.slowq[q]);
+            first = q - n;
         }
         __syncthreads();
     }
