@@ -933,11 +933,16 @@ static cudaError_t host_order(tlsph_ctx *ctx)
 {
     if (!ctx->reordered || !ctx->perm.empty()) return cudaSuccess;
     const size_t n = (size_t)ctx->N;
-    std::vector<int32_t> perm(n);
+    std::vector<int32_t> perm;
+    try {
+        perm.resize(n);
+        ctx->inv.resize(n);
+    } catch (const std::bad_alloc &) {
+        return cudaErrorMemoryAllocation;
+    }
     cudaError_t e = cudaMemcpyAsync(perm.data(), ctx->perm_dev, n * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return e;
-    ctx->inv.resize(n);
     for (size_t k = 0; k < n; ++k) ctx->inv[perm[k]] = (int32_t)k;
     ctx->perm.swap(perm);
     return cudaSuccess;

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(NBR_THREADS) k_nbr(const double *X, int64_t N,
                     const float r2f = ex * ex + ey * ey + ez * ez;
                     const int j = __float_as_int(c[u].w);
                     if (r2f > pf.hi || k0 + u >= e || j == (int)i) continue;
-                    if (r2f >= pf.lo) {
+                    if (!(r2f < pf.lo)) {
                         band[nband++][threadIdx.x] = j;
                         if (nband == NBR_BAND) {
                             n = test_band(X, i, rc2, &band[0][threadIdx.x], nband, o, n);
