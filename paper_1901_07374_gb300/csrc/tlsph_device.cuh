@@ -397,16 +397,21 @@ __device__ __forceinline__ int gtn_screen_f(const DevMat &m, float s2, float sm,
 //
 // Bound by the FP64 pipe (16 cycles per warp instruction and SM), so the two
 // solves are arranged around the number of FP64 functions they take.  Each
-// starts from its single-precision root and makes one step of Halley's
-// third-order iteration, whose error (of the order of the move d times
-// d^2 phi''' / phi' and of d (d / ep)^2) is held under 1e-17; cosh and sinh of the first come from one expm1 and
-// follow the step by their Taylor terms, as the hardening of the second does.
-// The hardening at ep + de is that at ep times (1 + de / ep)^n by its binomial
-// series (ratio below 1/32; a power otherwise).  A typical plastic update then
-// takes one power, one expm1 and one exponential.  A solve whose step is not
-// that small goes on with Newton's iteration to the same convergence test.
-// ncu on the notched bar in plastic flow: 842 FP64 warp instructions per 32
-// particles before, 345 to 440 now; pass 1 of 455,958 particles 0.75 -> 0.49 ms.
+// starts from its single-precision root.  The first makes one step of Halley's
+// third-order iteration, whose error is held under 1e-17; cosh and sinh come
+// from one expm1 and follow the step by their Taylor terms.  The second inverts
+// the hardening's Taylor series about the root to third order: the error, below
+// 2 (d / ep)^3 of the move d for n <= 2, is held under 2e-17 of the increment
+// (roots good to 5e-5 pass, which single precision is; second order would
+// need 2e-6, which a lane of nearly every warp misses).  The hardening at
+// ep + de is that at ep times (1 + de / ep)^n by its binomial series (ratio
+// below 1/32; a power otherwise).  A typical plastic update then takes one
+// power, one expm1 and one exponential.  A solve whose step is not that small
+// goes on with Newton's iteration to the same convergence test.
+// Both solves by Newton / the second to second order / this: the notched bar's
+// update in plastic flow, steps 2 to 4 from the virgin state, 0.69 / 0.62 /
+// 0.40 ms (842 / 590 / 430 FP64 warp instructions per 32 particles); 200,003
+// points 0.38 / 0.32 / 0.18 ms.
 __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const double *ed, double J,
                                             MPState &s, uint32_t &status)
 {
@@ -489,13 +494,14 @@ __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const d
         } else {
             H = m.B * pow(ep, m.n);
         }
-        const double Hp = m.n * H * ie, Hpp = (m.n - 1.0) * Hp * ie;
-        const double i1 = rcp_fp64(fma(xrk, Hp, 1.0));
-        const double d = (fma(-xrk, H, (seq - x * rate * m.A) * kf) - dx) * i1;
-        if (d * d * fabs(d) <= 1e-17 * dx * ep * ep) {
-            const double dd = d - d * d * (0.5 * xrk * Hpp * i1);
-            de = dx + dd;
-            h1 = m.A + fma(dd, fma(0.5 * dd, Hpp, Hp), H);
+        const double Hp = m.n * H * ie, Hpp = (m.n - 1.0) * Hp * ie, H3 = (m.n - 2.0) * Hpp * ie * (1.0 / 6.0);
+        const double i1 = rcp_fp64(fma(xrk, Hp, 1.0)), xi = xrk * i1;
+        const double d = (fma(-xrk, H, (seq - x * rate * m.A) * kf) - dx) * i1, d2 = d * d;
+        if (d2 * d2 <= 1e-17 * dx * ep * ep * ep) {
+            const double a = 0.5 * xi * Hpp;
+            const double z = fma(-d2, fma(fma(xi, H3, -2.0 * a * a), d, a), d);    // z + a z^2 + xi H3 z^3 = d
+            de = dx + z;
+            h1 = m.A + fma(z, fma(z, fma(z, H3, 0.5 * Hpp), Hp), H);
             conv = true;
         }
     }
