@@ -273,7 +273,8 @@ int tlsph_destroy(tlsph_ctx *ctx);
  * per 32 rows; 1 thread per row, two pairs in flight; 2 thread-per-row
  * gather + per-particle kernel; 3 thread per row, one pair in flight; 4, 7
  * and 8 thread per row, eight slots a turn, in blocks of 320 from 400,000
- * particles on whatever the plan's block size; 5 as 3 with registers capped
+ * particles on whatever the plan's block size (8 adds the products of two
+ * stress rows in the order x, y, z); 5 as 3 with registers capped
  * for eight resident blocks; 6 as 1 capped for seven resident blocks; block
  * size at most 128 for 4 to 8),
  * plan[3] its block size (multiples of 32 up to 256).  On contexts of less

@@ -1094,7 +1094,11 @@ __device__ __forceinline__ Row2 load_row2(const DevState &s, const MixConst &c, 
 // form once a turn took eight slots (1.02M particles: 0.553 against 0.548 ms).
 // IDX32 forms the record's index in 32 bits: 6 N records, N under 7e8, which a
 // mixed context's more than 700 bytes per particle imply on a device of 288 GB.
-template <bool HG, bool IDX32>
+// With XYZ, rows 0 and 1 of (A_j - A_i) X_ij add their products in the order
+// x, y, z, each rounding written out; otherwise in the compiler's.  The two
+// differ by FP32 rounding, which cancellation makes 2e-5 of the largest force on
+// the 1.02M-particle bar, so plan form 8 keeps its own order.
+template <bool HG, bool IDX32, bool XYZ>
 __device__ __forceinline__ void pair2(const DevState &s, const MixConst &c, const Row2 &w, int j, float qpad,
                                       float *acc)
 {
@@ -1111,8 +1115,14 @@ __device__ __forceinline__ void pair2(const DevState &s, const MixConst &c, cons
     const float gd = b2.y * g0;                    // V_j D_j W'/r
     acc[0] += gd * d.x; acc[1] += gd * d.y; acc[2] += gd * d.z;
     // (A_j - A_i) X_ij
-    const float t0 = (b0.x + w.nA0.x) * d.x + (b0.z + w.nA1.x) * d.y + (b1.x + w.nA2.x) * d.z;
-    const float t1 = (b0.y + w.nA0.y) * d.x + (b0.w + w.nA1.y) * d.y + (b1.y + w.nA2.y) * d.z;
+    float t0, t1;
+    if (XYZ) {
+        t0 = __fmaf_rn(b1.x + w.nA2.x, d.z, __fmaf_rn(b0.z + w.nA1.x, d.y, __fmul_rn(b0.x + w.nA0.x, d.x)));
+        t1 = __fmaf_rn(b1.y + w.nA2.y, d.z, __fmaf_rn(b0.w + w.nA1.y, d.y, __fmul_rn(b0.y + w.nA0.y, d.x)));
+    } else {
+        t0 = (b0.x + w.nA0.x) * d.x + (b0.z + w.nA1.x) * d.y + (b1.x + w.nA2.x) * d.z;
+        t1 = (b0.y + w.nA0.y) * d.x + (b0.w + w.nA1.y) * d.y + (b1.y + w.nA2.y) * d.z;
+    }
     const float t2 = fmaf(b2.x + w.nA22, d.z, fmaf(b1.w + w.nA21, d.y, (b1.z + w.nA20) * d.x));
     acc[3] += g * t0; acc[4] += g * t1; acc[5] += g * t2;
     if (HG) {
@@ -1149,7 +1159,7 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
         float acc[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-        for (int64_t p = p0 + lane; p < p1; p += 32) pair2<HG, false>(s, c, w, s.col[p], 0.0f, acc);
+        for (int64_t p = p0 + lane; p < p1; p += 32) pair2<HG, false, false>(s, c, w, s.col[p], 0.0f, acc);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             if (!HG && k >= 6) continue;
@@ -1162,7 +1172,7 @@ __global__ void __launch_bounds__(MIX_THREADS) k_pass2_mixed(DevState s, MixCons
 }
 
 // pass-2 pair sums of row i over its slots, U pairs in flight
-template <bool HG, int U, int L = 1, int TU = U, bool IDX32 = false>
+template <bool HG, int U, int L = 1, int TU = U, bool IDX32 = false, bool XYZ = false>
 __device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c, int64_t i, float *acc, int sub = 0)
 {
     const Row2 w = load_row2<HG>(s, c, i);
@@ -1170,7 +1180,7 @@ __device__ __forceinline__ void gather2_row(const DevState &s, const MixConst &c
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
     for_slots<U, L, TU>(s, i, sub, [&](const int *j, const float *wm, int, auto count) {
 #pragma unroll
-        for (int u = 0; u < decltype(count)::value; ++u) pair2<HG, IDX32>(s, c, w, j[u], wm[u], acc);
+        for (int u = 0; u < decltype(count)::value; ++u) pair2<HG, IDX32, XYZ>(s, c, w, j[u], wm[u], acc);
     });
 }
 
@@ -1237,21 +1247,21 @@ __global__ void __launch_bounds__(128, 7) k_pass2_mixed_tc7(DevState s, MixConst
 // of 128 these two are the better ones, 0.549 against 0.555); blocks of 160 /
 // 384 / 640 0.538 / 0.545 / 0.586; packed FP32x2 stress rows 0.553 in blocks of 128.
 constexpr int64_t PASS2_WIDE_FROM = 400000;
-template <bool HG, bool WIDE>
+template <bool HG, bool WIDE, bool XYZ>
 __global__ void __launch_bounds__(WIDE ? 320 : 128, WIDE ? 2 : 5) k_pass2_mixed_tc(DevState s, MixConst c)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.N) return;
     float acc[9];
-    gather2_row<HG, 8, 1, WIDE ? 1 : 2, WIDE>(s, c, i, acc);
+    gather2_row<HG, 8, 1, WIDE ? 1 : 2, WIDE, XYZ>(s, c, i, acc);
     epi2_mixed<HG>(s, c, i, acc);
 }
 
-template <bool HG>
+template <bool HG, bool XYZ>
 static void launch_pass2_tc(const DevState &s, const MixConst &c, int block, cudaStream_t st)
 {
-    if (s.N >= PASS2_WIDE_FROM) k_pass2_mixed_tc<HG, true><<<nb(s.N, 320), 320, 0, st>>>(s, c);
-    else k_pass2_mixed_tc<HG, false><<<nb(s.N, block), block, 0, st>>>(s, c);
+    if (s.N >= PASS2_WIDE_FROM) k_pass2_mixed_tc<HG, true, XYZ><<<nb(s.N, 320), 320, 0, st>>>(s, c);
+    else k_pass2_mixed_tc<HG, false, XYZ><<<nb(s.N, block), block, 0, st>>>(s, c);
 }
 
 // registers capped for eight blocks of 128 to an SM: 1.02M particles 0.336 -> 0.326 ms with the update
@@ -1658,7 +1668,7 @@ int mixed_slow_grid()
 //           2 = thread-per-row gather + per-particle kernel;  3 = warp-per-32-rows gather + per-particle kernel;
 //           4 = as 2 with four pairs in flight per thread;  5 = as 4 with the weights W'/r from the per-slot table
 //   pass 2: 0 = warp per 32 rows;  1 = thread per row;  2 = thread-per-row gather + per-particle kernel;
-//           3 = thread per row, one pair in flight;  4, 7, 8 = thread per row, eight slots a turn;
+//           3 = thread per row, one pair in flight;  4, 7, 8 = thread per row, eight slots a turn (8: stress rows in the order x, y, z);
 //           5 = as 3 with registers capped for 8 blocks of 128;  6 = as 1 with registers capped for 7 blocks of 128
 // block sizes are multiples of 32 up to 256 (128 for the fused warp forms and pass-2 forms 4 to 8).
 // Pass-1 forms 4 and 5 and pass-2 form 4 share a row between several lanes on small contexts (row_lanes).
@@ -1718,8 +1728,10 @@ cudaError_t launch_step_mixed(tlsph_ctx &ctx, int64_t step_index, cudaStream_t s
         if (hg) k_pass2_mixed_tc7<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_tc7<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
     } else if (v2 == 4 || v2 == 7 || v2 == 8) {
-        if (hg) launch_pass2_tc<true>(s, c, b2, st);
-        else launch_pass2_tc<false>(s, c, b2, st);
+        if (hg && v2 == 8) launch_pass2_tc<true, true>(s, c, b2, st);
+        else if (hg) launch_pass2_tc<true, false>(s, c, b2, st);
+        else if (v2 == 8) launch_pass2_tc<false, true>(s, c, b2, st);
+        else launch_pass2_tc<false, false>(s, c, b2, st);
     } else if (v2 == 5) {
         if (hg) k_pass2_mixed_t1c<true><<<nb(s.N, b2), b2, 0, st>>>(s, c);
         else k_pass2_mixed_t1c<false><<<nb(s.N, b2), b2, 0, st>>>(s, c);
@@ -1803,11 +1815,11 @@ __device__ __forceinline__ int batch_find(const int64_t *blk0, int n, int64_t w)
 // the compiler fuses).
 //   pass-1 gather:        (8, 4)  (6, 4)  (10, 4)  (8, 2)  (8, 4) with the members' per-slot weight tables
 //   per-particle update:  5  4  3
-//   pass 2:               (2 blocks of 320, 8)  (6, 2)  (5, 8)  (8, 1)  (5, 2)
+//   pass 2:               (2 blocks of 320, 8)  (6, 2)  (5, 8)  (8, 1)  (5, 2) with the rows' order of plan form 8
 const int BATCH_VARIANTS[BATCH_KINDS] = { 5, 3, 5 };
 
 // TAB: the pass-1 gather reads the members' per-slot weight tables (members
-// must hold one)
+// must hold one); pass 2 adds the stress rows' products in the order x, y, z
 template <int KIND, bool HG, int MINB, int U, bool TAB = false, int BLOCK = 128>
 __global__ void __launch_bounds__(BLOCK, MINB) k_batch(BatchHdr *hdr, const BatchSlot *slots)
 {
@@ -1852,7 +1864,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_batch(BatchHdr *hdr, const Batc
                     epi1_mixed(st, c, i, mm);
                 } else {                    // pass 2
                     float acc[9];
-                    gather2_row<HG, U, 1, U == 8 ? (WB ? 1 : 2) : U, WB == 1>(st, c, i, acc);
+                    gather2_row<HG, U, 1, U == 8 ? (WB ? 1 : 2) : U, WB == 1, TAB>(st, c, i, acc);
                     epi2_mixed<HG>(st, c, i, acc);
                 }
             }
@@ -1943,7 +1955,7 @@ struct BatchKernel {
             case 1: return k_batch<2, HG, 6, 2>;
             case 2: return k_batch<2, HG, 5, 8>;
             case 3: return k_batch<2, HG, 8, 1>;
-            case 4: return k_batch<2, HG, 5, 2>;
+            case 4: return k_batch<2, HG, 5, 2, true>;
             default: return k_batch<2, HG, 2, 8, false, BATCH_WIDE>;
             }
         }

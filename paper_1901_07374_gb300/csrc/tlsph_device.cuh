@@ -410,7 +410,7 @@ __device__ __forceinline__ int gtn_screen_f(const DevMat &m, float s2, float sm,
 // goes on with Newton's iteration to the same convergence test.
 // Both solves by Newton / the second to second order / this: the notched bar's
 // update in plastic flow, steps 2 to 4 from the virgin state, 0.69 / 0.62 /
-// 0.40 ms (842 / 590 / 430 FP64 warp instructions per 32 particles); 200,003
+// 0.40 ms (842 / 690 / 430 FP64 warp instructions per 32 particles); 200,003
 // points 0.38 / 0.32 / 0.18 ms.
 __device__ __forceinline__ double gtn_update(const DevMat &m, double dt, const double *ed, double J,
                                             MPState &s, uint32_t &status)
