@@ -80,12 +80,13 @@ def algorithmic_bytes(N: int, nnz: int, precision: str, list_words: int | None =
 # precision, pass, plan form of that pass) and stamped with the digest of the
 # CUDA sources they were captured from: a figure is reported only while the
 # sources are unchanged (otherwise `traffic` is null until the next capture).
-TRAFFIC_SOURCES = "e6cc72b91479d63571156f6acb48bdfce3161c74b68082d8707498a63375bcbc"
+TRAFFIC_SOURCES = "434c623367b2d71eccef70d40af0cb7a07ab295d707cdf6591bf0c32447b6e72"
 TRAFFIC = {
-    ("tensile_bar_jc_40x40x640", "mixed", "pass1", 4): 597210624,    # k_gather1_mixed_t4 + k_epi1_mixed + k_epi1_slow
-    ("tensile_bar_jc_40x40x640", "mixed", "pass1", 5): 1098680832,   # k_gather1_mixed_t4w (weight table) + the same
-    ("tensile_bar_jc_40x40x640", "mixed", "pass2", 7): 327032320,    # k_pass2_mixed_tc5
-    ("tensile_bar_jc_40x40x640", "mixed", "pass2", 8): 327364864,    # k_pass2_mixed_tc5p
+    ("tensile_bar_jc_40x40x640", "mixed", "pass1", 4): 597435392,    # k_gather1_mixed_t4 + k_epi1_mixed + k_epi1_slow
+    ("tensile_bar_jc_40x40x640", "mixed", "pass1", 5): 1098909440,   # k_gather1_mixed_t4w (weight table) + the same
+    ("tensile_bar_jc_40x40x640", "mixed", "pass2", 4): 327330048,    # k_pass2_mixed_tc
+    ("tensile_bar_jc_40x40x640", "mixed", "pass2", 7): 327330048,
+    ("tensile_bar_jc_40x40x640", "mixed", "pass2", 8): 327294720,
 }
 
 
@@ -265,12 +266,15 @@ def field_scales(w) -> dict:
     return dict(U=L, V=v, F=1.0, SIGMA=s, STRESS_DEV=s, EPSP=1e-3, DINIT=1e-3, DAMAGE=1e-3, FORCE=s * L * L)
 
 
-def launches_per_step(plan) -> int:
-    """Kernels one step launches: FP64 path 2; mixed plans 1 or 2 per pass plus
-    the FP64-update kernel of pass 1."""
+def launches_per_step(plan, n: int, hourglass: bool) -> int:
+    """Kernels one step of n particles launches: FP64 path one per pass and one
+    for the hourglass vectors; mixed plans 1 or 2 per pass plus the FP64-update
+    kernel of pass 1, which forms 4 and 5 fuse with the others on contexts of
+    less than 50,000 particles."""
     if not plan:
-        return 2
-    return (2 if plan[0] >= 2 else 1) + 1 + (2 if plan[2] == 2 else 1)
+        return 3 if hourglass else 2
+    fused = plan[0] in (4, 5) and n < 50000
+    return (1 if fused else (2 if plan[0] >= 2 else 1) + 1) + (2 if plan[2] == 2 else 1)
 
 
 def field_errors(sim, ref: dict, sc: dict) -> dict:
@@ -577,7 +581,7 @@ def run_ours(args, rank: int, world: int, dist):
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64" if args.precision == "fp64" else "f32+f64",
             "data": "synthetic (seeded jittered lattice)", "config": cfg,
-            "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches_per_step(r.get("plan")) * args.steps,
+            "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches_per_step(r.get("plan"), N, w.hg_alpha != 0.0) * args.steps,
             "clocks": r["clocks"]}
     print(json.dumps(line), flush=True)
 
@@ -691,13 +695,14 @@ def measure_batched(tlsph, torch, ws, steps: int, warmup: int, stream, fp64_one_
     ms_seq = e0.elapsed_time(e1)
     for s in sims:
         s.sync()
+    one_by_one = sum(launches_per_step(autotune.DEFAULT, s.N, ws[0].hg_alpha != 0.0) for s in sims)
     b.close()
     for s in sims:
         s.close()
     out = {"specimens": len(ws), "particles": N, "pairs_per_step": nnz, "set_up_s": setup,
            "ms_per_step": ms / steps, "value": nnz * steps / (ms * 1e-3),
            "one_by_one_value": nnz * steps / (ms_seq * 1e-3), "one_by_one_ms_per_step": ms_seq / steps,
-           "kernel_launches_per_step": {"batched": 5, "one_by_one": 4 * len(ws)},
+           "kernel_launches_per_step": {"batched": 5, "one_by_one": one_by_one},
            "list_words": sum(x["words"] for x in lays), "launch_shape": list(shape), "tune_s": tune_s,
            "clocks": clocks}
     if fp64_one_by_one:
