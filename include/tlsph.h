@@ -198,7 +198,11 @@ int tlsph_create(const tlsph_config *cfg, int64_t N, const double *X, const doub
 
 /* Set material `mat_id` (Sec. 4-5 constants).  Every material referenced by
  * mat_id must be set before the first tlsph_step.  Setting a GTN material
- * before the first step also sets D = q1 f*(f0) on its particles. */
+ * before the first step also sets D = q1 f*(f0) on its particles.  Once every
+ * material in use is set, an FP64 context in library-owned memory also keeps
+ * a table of 52 bytes per neighbour pair, unless that is more than a quarter
+ * of the free device memory (its steps then form the same terms in place, to
+ * the same bits). */
 int tlsph_set_material(tlsph_ctx *ctx, int mat_id, const tlsph_material *mat);
 
 /* Enqueue nsteps time steps on the context's stream (asynchronous; errors of
